@@ -393,6 +393,26 @@ pced_status make_tmap_2d(CUtensorMap* map, const void* base, uint64_t rows, uint
                          uint32_t box_cols, bool l2_promote_256);
 pced_status make_tmap_kv(CUtensorMap* map, const void* base, uint64_t rows, uint32_t D, uint32_t box_rows);
 
+// Launch a kernel as a programmatic dependent of the stream's previous kernel.
+// Every such kernel calls pdl_wait() in all of its threads' CTAs before it
+// touches global memory, so it sees what every earlier launch wrote; only its
+// launch, and what it does before the wait, overlap the previous kernel.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+                       A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // carve consecutive 256-byte aligned regions out of a workspace

@@ -2,19 +2,35 @@
 // path behind pced_contrastive_select).
 //   shat_k(v) = (1 + beta_k) lp_k(v) - beta_k lp_0(v) + gamma log r_k,  k = 1..N
 //   y = argmax_v max_k shat_k(v)
-// Pass 1: one CTA per (vocabulary chunk, query) scans its tokens, taking the
-// max over experts per token and the best token of the chunk.  Pass 2: one
-// CTA per query reduces the chunk records.  Ties: highest score, then lowest
-// token id, then lowest expert index (the amateur, row 0, never competes).
+// Pass 1: a cluster of SEL_CLUSTER CTAs per (SEL_CHUNK tokens, query) takes the
+// max over experts per token and the chunk's best token; pass 2: one warp per
+// query reduces the chunk records.  Ties: highest score, then lowest token id,
+// then lowest expert index (the amateur, row 0, never competes).
+//
+// What bounds it: a few MB per query, so latency until the rows are tens of
+// MB and the loads after that.  One CTA per 4096 tokens left most SMs idle
+// (32 CTAs at V = 128256, one query) and each thread waited for one load at a
+// time: 28.6 us + 2.8 us of a second launch for 9 rows, 128 us for 16 x 17
+// rows.  Now a thread has SEL_TOK tokens of SEL_ROWS experts in flight, four
+// CTAs share a chunk (their bests meet in the first one's shared memory, so
+// the workspace still holds one record per SEL_CHUNK tokens), and the second
+// kernel is resident before the first one ends (programmatic launch).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "common.cuh"
 
 namespace pced {
 
+namespace cg = cooperative_groups;
+
 constexpr int SEL_THREADS = 256;
-constexpr int SEL_CHUNK = 4096;
+constexpr int SEL_TOK = 4;      // tokens of a thread
+constexpr int SEL_ROWS = 4;     // expert rows loaded at a time
+constexpr int SEL_CLUSTER = 4;  // CTAs per chunk record
+constexpr int SEL_CHUNK = SEL_CLUSTER * SEL_THREADS * SEL_TOK;
 constexpr int SEL_MAX_N = 255;
+constexpr int SEL_NONE = 0x7fffffff;
 
 struct Cand {
   float s;
@@ -34,55 +50,91 @@ __device__ __forceinline__ Cand warp_best(Cand c) {
   }
   return c;
 }
-__device__ __forceinline__ Cand block_best(Cand c) {
-  __shared__ Cand red[SEL_THREADS / 32];
-  c = warp_best(c);
-  const int tid = threadIdx.x;
-  if ((tid & 31) == 0) red[tid >> 5] = c;
-  __syncthreads();
-  if (tid < 32) {
-    Cand d = tid < SEL_THREADS / 32 ? red[tid] : Cand{-INFINITY, 0x7fffffff, 0x7fffffff};
-    d = warp_best(d);
-    if (tid == 0) red[0] = d;
-  }
-  __syncthreads();
-  return red[0];
-}
 
-__global__ void __launch_bounds__(SEL_THREADS)
+__global__ void __cluster_dims__(SEL_CLUSTER, 1, 1) __launch_bounds__(SEL_THREADS)
     select_dense_kernel(const float* __restrict__ lp, const float* __restrict__ beta, const float* __restrict__ r,
                         float gamma, int N, int V, Cand* rec) {
+  cg::cluster_group cluster = cg::this_cluster();
   const int b = blockIdx.y, tid = threadIdx.x, n1 = N + 1;
   __shared__ float bt[SEL_MAX_N], bias[SEL_MAX_N];
+  __shared__ Cand wbest[SEL_THREADS / 32], cbest[SEL_CLUSTER];
+  cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
+  pdl_launch_dependents();
+  pdl_wait();
   for (int k = tid; k < N; k += SEL_THREADS) {
     bt[k] = beta[b * N + k];
     bias[k] = gamma * logf(fminf(fmaxf(r[b * N + k], 1e-8f), 1.0f));
   }
-  __syncthreads();
   const float* lp0 = lp + (int64_t)b * n1 * V;
-  Cand best{-INFINITY, 0x7fffffff, 0x7fffffff};
-  const int v0 = blockIdx.x * SEL_CHUNK, v1 = min(V, v0 + SEL_CHUNK);
-  for (int v = v0 + tid; v < v1; v += SEL_THREADS) {
-    const float a0 = lp0[v];
-    for (int k = 1; k <= N; ++k) {
-      const float x = (1.f + bt[k - 1]) * lp0[(int64_t)k * V + v] - bt[k - 1] * a0 + bias[k - 1];
-      const Cand c{x, v, k};
-      if (cand_better(c, best)) best = c;
+  const int v0 = blockIdx.x * (SEL_THREADS * SEL_TOK) + tid;
+  float a0[SEL_TOK], s[SEL_TOK];
+  int kk[SEL_TOK];
+#pragma unroll
+  for (int j = 0; j < SEL_TOK; ++j) {
+    const int v = v0 + j * SEL_THREADS;
+    a0[j] = v < V ? lp0[v] : 0.f;
+    s[j] = -INFINITY;
+    kk[j] = SEL_NONE;
+  }
+  __syncthreads();
+  for (int k0 = 1; k0 <= N; k0 += SEL_ROWS) {
+    float x[SEL_ROWS][SEL_TOK];
+#pragma unroll
+    for (int u = 0; u < SEL_ROWS; ++u)
+#pragma unroll
+      for (int j = 0; j < SEL_TOK; ++j) {
+        const int v = v0 + j * SEL_THREADS;
+        x[u][j] = k0 + u <= N && v < V ? lp0[(int64_t)(k0 + u) * V + v] : 0.f;
+      }
+#pragma unroll
+    for (int u = 0; u < SEL_ROWS; ++u) {
+      const int k = k0 + u;
+      if (k > N) break;
+#pragma unroll
+      for (int j = 0; j < SEL_TOK; ++j) {
+        const float y = (1.f + bt[k - 1]) * x[u][j] - bt[k - 1] * a0[j] + bias[k - 1];
+        if (y > s[j] || (y == s[j] && k < kk[j])) {  // k rises: a tie keeps the lower expert
+          s[j] = y;
+          kk[j] = k;
+        }
+      }
     }
   }
-  best = block_best(best);
-  if (tid == 0) rec[(int64_t)b * gridDim.x + blockIdx.x] = best;
+  Cand best{-INFINITY, SEL_NONE, SEL_NONE};
+#pragma unroll
+  for (int j = 0; j < SEL_TOK; ++j) {
+    const int v = v0 + j * SEL_THREADS;
+    const Cand c{s[j], v, kk[j]};
+    if (v < V && kk[j] != SEL_NONE && cand_better(c, best)) best = c;
+  }
+  best = warp_best(best);
+  if ((tid & 31) == 0) wbest[tid >> 5] = best;
+  __syncthreads();
+  if (tid < 32) {
+    best = warp_best(tid < SEL_THREADS / 32 ? wbest[tid] : Cand{-INFINITY, SEL_NONE, SEL_NONE});
+  }
+  cluster.barrier_wait();
+  if (tid == 0) *cluster.map_shared_rank(cbest + cluster.block_rank(), 0) = best;
+  cluster.sync();
+  if (tid == 0 && cluster.block_rank() == 0) {
+#pragma unroll
+    for (int i = 1; i < SEL_CLUSTER; ++i)
+      if (cand_better(cbest[i], best)) best = cbest[i];
+    rec[(int64_t)b * (gridDim.x / SEL_CLUSTER) + blockIdx.x / SEL_CLUSTER] = best;
+  }
 }
 
-__global__ void __launch_bounds__(SEL_THREADS)
+__global__ void __launch_bounds__(32)
     select_reduce_kernel(const Cand* rec, int nchunks, int32_t* token, int32_t* expert, float* score) {
   const int b = blockIdx.x;
-  Cand best{-INFINITY, 0x7fffffff, 0x7fffffff};
-  for (int i = threadIdx.x; i < nchunks; i += SEL_THREADS) {
+  pdl_wait();
+  Cand best{-INFINITY, SEL_NONE, SEL_NONE};
+#pragma unroll 4
+  for (int i = threadIdx.x; i < nchunks; i += 32) {
     const Cand c = rec[(int64_t)b * nchunks + i];
     if (cand_better(c, best)) best = c;
   }
-  best = block_best(best);
+  best = warp_best(best);
   if (threadIdx.x == 0) {
     token[b] = best.v;
     expert[b] = best.k;
@@ -118,11 +170,10 @@ extern "C" pced_status pced_contrastive_select(const float* logprobs, const floa
   Carver cv((char*)workspace + 256);
   Cand* rec = cv.take<Cand>((size_t)B * nchunks);
   cudaStream_t s = (cudaStream_t)stream;
-  select_dense_kernel<<<dim3(nchunks, B), SEL_THREADS, 0, s>>>(logprobs, beta, r, gamma, N, V, rec);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(select_dense_kernel, dim3(nchunks * SEL_CLUSTER, B), SEL_THREADS, 0, s, logprobs, beta, r,
+                             gamma, N, V, rec);
   if (e != cudaSuccess) return cuda_status(e, "select launch");
-  select_reduce_kernel<<<B, SEL_THREADS, 0, s>>>(rec, nchunks, token, expert, score);
-  e = cudaGetLastError();
+  e = launch_pdl(select_reduce_kernel, dim3(B), 32, 0, s, (const Cand*)rec, nchunks, token, expert, score);
   if (e != cudaSuccess) return cuda_status(e, "select reduce launch");
   return PCED_OK;
 }

@@ -46,6 +46,13 @@ def test_n32_no_contrast(cuda_ok):
     run_case(2, 32, 3000, 4, beta_val=0.0)
 
 
+@pytest.mark.parametrize("B,N,V", [(1, 1, 1), (2, 3, 255), (1, 4, 1024), (2, 5, 1025), (1, 9, 4095), (3, 4, 4097),
+                                   (1, 255, 8191)])
+def test_edges_of_chunks_and_expert_batches(cuda_ok, B, N, V):
+    """Vocabularies around a thread block's 1024 tokens and a record's 4096, experts around the batch of four rows."""
+    run_case(B, N, V, 100 + N + V)
+
+
 def test_exact_ties_follow_lowest_token_then_expert(cuda_ok):
     import paper_2601_08670_gb300 as pced
     V, N = 10, 3
