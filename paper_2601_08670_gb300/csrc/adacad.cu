@@ -5,88 +5,119 @@
 // expert's next-token distribution p_k = exp(lp_k) and the amateur's
 // p_0 = exp(lp_0):
 //   beta[b][k-1] = 1/2 sum_v [ p_k log2(p_k / m) + p_0 log2(p_0 / m) ],  m = (p_k + p_0) / 2,
-// in [0, 1].  CTAs of 8192 vocabulary entries per (expert, query) stream both
-// rows once; each term uses log m = logaddexp(lp_k, lp_0) - ln 2 in fp32 and
-// is summed in fp64 in a fixed order (thread t takes v = t, t + 256, ... of
-// its chunk, then a fixed tree, then the chunks in order by the last CTA of
-// the pair to finish), so the result does not depend on timing.
+// in [0, 1].  With hi / lo the larger and smaller of the two log-probabilities
+// and e = exp(lo - hi), a term is
+//   exp(hi) [ q + e (q + lo - hi) ],  q = ln 2 - log1p(e) = log(p_hi / m),
+// in fp32, without the rounding of a logarithm of the size of hi.
+//
+// What bounds it: two exp and one log1p per entry and expert (and, past the
+// L2, the rows).  A cluster of ADA_CLUSTER CTAs takes one (expert, query): the
+// cluster's sums meet in the first CTA's shared memory, so there is no scratch,
+// no counter to clear and no second pass.  (One CTA per 2048 entries left the
+// last one to add 63 chunk sums one load after the other: 14.8 us for 8
+// experts of 128256 entries beside a memset; 180 us for 16 x 16.)
+//
+// Sums are held as an unevaluated pair of fp32 numbers (error-free addition,
+// about 48 bits) and rounded once from fp64 at the end: this chip adds 64-bit
+// numbers at 1/64 of the fp32 rate, so one fp64 conversion and addition per
+// entry cost more than the entry's exponentials.  The order is fixed (thread,
+// then xor trees over lanes and warps, then the CTAs in order), so the result
+// does not depend on timing.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "adacad.cuh"
 
 namespace pced {
 
-constexpr int ADA_THREADS = 256;
-constexpr int ADA_CHUNK = 2048;  // vocabulary entries per CTA (about 500 CTAs at llama8: every SM busy)
+namespace cg = cooperative_groups;
 
-int32_t adacad_chunks(int32_t V) { return (V + ADA_CHUNK - 1) / ADA_CHUNK; }
+constexpr int ADA_THREADS = 1024;
+constexpr int ADA_CLUSTER = 8;
+constexpr int ADA_UNROLL = 4;  // entries of a thread in flight
 
-// grid (chunks, N, B): CTA (c, k-1, b) sums the terms of v in chunk c; the
-// last CTA of (b, k) to finish adds the chunk sums in chunk order
-__global__ void __launch_bounds__(ADA_THREADS) adacad_beta_kernel(const float* lp, int32_t N, int32_t V, float* beta,
-                                                                  double* part, int* cnt, int* reset_ctr) {
-  const int c = blockIdx.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
-  const int nch = gridDim.x;
-  if (reset_ctr && c == 0 && k == 1 && b == 0 && tid == 0) *reset_ctr = 0;
+// an fp32 pair s + c, |c| below half an ulp of s times the terms added
+struct Pair {
+  float s, c;
+};
+// (a + b) exactly as sum + error (Knuth's two-sum; the _rn forms keep the
+// compiler from contracting it)
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float y = __fadd_rn(a, b), z = __fsub_rn(y, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(y, z)), __fsub_rn(b, z));
+  return y;
+}
+__device__ __forceinline__ void pair_add(Pair& p, float t) {
+  float e;
+  p.s = two_sum(p.s, t, e);
+  p.c = __fadd_rn(p.c, e);
+}
+__device__ __forceinline__ Pair pair_merge(Pair p, Pair q) {
+  float e;
+  const float s = two_sum(p.s, q.s, e);
+  return Pair{s, __fadd_rn(__fadd_rn(p.c, q.c), e)};
+}
+__device__ __forceinline__ Pair warp_pair(Pair p) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    p = pair_merge(p, Pair{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.c, o)});
+  return p;
+}
+
+__device__ __forceinline__ float jsd_term(float a, float b) {
+  const float ln2 = 0.69314718055994531f;
+  const float hi = fmaxf(a, b), lo = fminf(a, b);
+  if (hi == -INFINITY) return 0.f;  // both probabilities are 0
+  const float d = lo - hi, e = expf(d), q = ln2 - log1pf(e);
+  return expf(hi) * (lo == -INFINITY ? q : q + e * (q + d));
+}
+
+// grid (ADA_CLUSTER, N, B), one cluster per (k - 1, b)
+__global__ void __cluster_dims__(ADA_CLUSTER, 1, 1) __launch_bounds__(ADA_THREADS)
+    adacad_beta_kernel(const float* __restrict__ lp, int32_t N, int32_t V, float* beta, int* reset_ctr) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = blockIdx.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
+  __shared__ Pair wsum[ADA_THREADS / 32], csum[ADA_CLUSTER];
+  cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
+  pdl_launch_dependents();
+  pdl_wait();
+  if (reset_ctr && rank == 0 && k == 1 && b == 0 && tid == 0) *reset_ctr = 0;
   const float* l0 = lp + (int64_t)b * (N + 1) * V;
   const float* lk = l0 + (int64_t)k * V;
-  const float ln2 = 0.69314718055994531f;
-  const int v1 = min(V, (c + 1) * ADA_CHUNK);
-  double acc = 0.0;
-  for (int v = c * ADA_CHUNK + tid; v < v1; v += ADA_THREADS) {
-    const float a = lk[v], cc = l0[v];
-    const float hi = fmaxf(a, cc), lo = fminf(a, cc);
-    if (hi == -INFINITY) continue;  // p_k = p_0 = 0
-    const float lm = hi + log1pf(expf(lo - hi)) - ln2;  // log of the midpoint
-    float t = 0.f;
-    if (a > -INFINITY) t += expf(a) * (a - lm);
-    if (cc > -INFINITY) t += expf(cc) * (cc - lm);
-    acc += (double)t;
-  }
+  const int per = (int)(((int64_t)V + ADA_CLUSTER - 1) / ADA_CLUSTER);
+  const int64_t v0 = (int64_t)rank * per, v1 = min((int64_t)V, v0 + per);
+  Pair acc{0.f, 0.f};
+  for (int64_t v = v0 + tid; v < v1; v += ADA_UNROLL * ADA_THREADS) {
+    float x[ADA_UNROLL], y[ADA_UNROLL];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  __shared__ double red[ADA_THREADS / 32];
-  __shared__ int last;
-  if ((tid & 31) == 0) red[tid >> 5] = acc;
-  __syncthreads();
-  const int64_t bk = (int64_t)b * N + (k - 1);
-  if (tid == 0) {
-    double s = 0.0;
-    for (int w = 0; w < ADA_THREADS / 32; ++w) s += red[w];
-    part[bk * nch + c] = s;
-    __threadfence();
-    last = atomicAdd(cnt + bk, 1) == nch - 1;
-    if (last) {
-      __threadfence();
-      double tot = 0.0;
-      for (int j = 0; j < nch; ++j) tot += __ldcg(part + bk * nch + j);
-      beta[bk] = (float)(0.5 * tot / 0.69314718055994531);
-      cnt[bk] = 0;
+    for (int u = 0; u < ADA_UNROLL; ++u) {
+      const bool in = v + u * ADA_THREADS < v1;
+      x[u] = in ? lk[v + u * ADA_THREADS] : -INFINITY;
+      y[u] = in ? l0[v + u * ADA_THREADS] : -INFINITY;
     }
+#pragma unroll
+    for (int u = 0; u < ADA_UNROLL; ++u) pair_add(acc, jsd_term(x[u], y[u]));
+  }
+  acc = warp_pair(acc);
+  if ((tid & 31) == 0) wsum[tid >> 5] = acc;
+  __syncthreads();
+  if (tid < 32) acc = warp_pair(wsum[tid]);
+  cluster.barrier_wait();
+  if (tid == 0) *cluster.map_shared_rank(csum + rank, 0) = acc;
+  cluster.sync();
+  if (rank == 0 && tid == 0) {
+    Pair t = csum[0];
+    for (int i = 1; i < ADA_CLUSTER; ++i) t = pair_merge(t, csum[i]);
+    beta[(int64_t)b * N + k - 1] = (float)(((double)t.s + (double)t.c) * 0.72134752044448170);  // 1 / (2 ln 2)
   }
 }
 
-size_t adacad_scratch_bytes(int32_t B, int32_t N, int32_t V) {
-  pced_host::Carver c(nullptr);
-  c.take<double>((size_t)B * N * adacad_chunks(V));
-  c.take<int>((size_t)B * N);
-  return c.used();
-}
-
-cudaError_t adacad_beta_launch(const float* lp, int32_t B, int32_t N, int32_t V, float* beta, void* scratch,
-                               int* reset_ctr, cudaStream_t stream) {
-  pced_host::Carver cv(scratch);
-  double* part = cv.take<double>((size_t)B * N * adacad_chunks(V));
-  int* cnt = cv.take<int>((size_t)B * N);
-  adacad_beta_kernel<<<dim3(adacad_chunks(V), N, B), ADA_THREADS, 0, stream>>>(lp, N, V, beta, part, cnt,
-                                                                                reset_ctr);
+cudaError_t adacad_beta_launch(const float* lp, int32_t B, int32_t N, int32_t V, float* beta, int* reset_ctr, bool pdl,
+                               cudaStream_t stream) {
+  const dim3 grid(ADA_CLUSTER, N, B);
+  if (pdl) return pced_host::launch_pdl(adacad_beta_kernel, grid, ADA_THREADS, 0, stream, lp, N, V, beta, reset_ctr);
+  adacad_beta_kernel<<<grid, ADA_THREADS, 0, stream>>>(lp, N, V, beta, reset_ctr);
   return cudaGetLastError();
-}
-
-int* adacad_counters(void* scratch, int32_t B, int32_t N, int32_t V) {
-  pced_host::Carver cv(scratch);
-  cv.take<double>((size_t)B * N * adacad_chunks(V));
-  return cv.take<int>((size_t)B * N);
 }
 
 }  // namespace pced
@@ -96,7 +127,12 @@ using namespace pced_host;
 
 extern "C" size_t pced_adacad_beta_workspace_size(int32_t B, int32_t N, int32_t V) {
   if (B < 1 || N < 1 || V < 1) return 0;
-  return adacad_scratch_bytes(B, N, V);
+  // the kernel needs no scratch; the size that callers allocate by stays (8
+  // bytes for each 2048 entries of an expert, 4 for each expert)
+  Carver c(nullptr);
+  c.take<double>((size_t)B * N * (((size_t)V + 2047) / 2048));
+  c.take<int>((size_t)B * N);
+  return c.used();
 }
 
 extern "C" pced_status pced_adacad_beta(const float* logprobs, int32_t B, int32_t N, int32_t V, float* beta,
@@ -110,9 +146,7 @@ extern "C" pced_status pced_adacad_beta(const float* logprobs, int32_t B, int32_
     return fail(PCED_ERR_WORKSPACE, "pced_adacad_beta: workspace too small or misaligned");
   if (num_sms() <= 0) return fail(PCED_ERR_NO_DEVICE, "pced_adacad_beta: no CUDA device");
   cudaStream_t s = (cudaStream_t)stream;
-  // the per-(query, expert) arrival counters start at zero (the kernel leaves them at zero)
-  cudaError_t e = cudaMemsetAsync(adacad_counters(workspace, B, N, V), 0, sizeof(int) * (size_t)B * N, s);
-  if (e == cudaSuccess) e = adacad_beta_launch(logprobs, B, N, V, beta, workspace, nullptr, s);
+  const cudaError_t e = adacad_beta_launch(logprobs, B, N, V, beta, nullptr, true, s);
   if (e != cudaSuccess) return cuda_status(e, "pced_adacad_beta launch");
   return PCED_OK;
 }

@@ -7,7 +7,8 @@
 //   reranker:                 r_rer = clip(sigmoid(z), 0, 1 - eps)
 //   fusion:                   r = 2 r_ret r_rer / (r_ret + r_rer + eps)   (harmonic mean, appendix form)
 // Elementwise, evaluated in fp64 and rounded to fp32 once.  Runs once per
-// query (not per token); a few hundred scores at most.
+// query (not per token); a few hundred scores at most, so all of it is launch
+// latency, which the next kernel's launch overlaps (programmatic launch).
 #include <math.h>
 
 #include "common.cuh"
@@ -21,6 +22,8 @@ __device__ __forceinline__ double rel_clip(double x, double eps) { return x < 0.
 __global__ void __launch_bounds__(REL_THREADS) relevance_kernel(const float* s, int32_t mode, const float* z,
                                                                 int32_t n, double eps, float* r) {
   const int k = blockIdx.x * REL_THREADS + threadIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
   if (k >= n) return;
   const double sk = s[k];
   const double rr = mode == 0 ? rel_clip((sk + 1.0) * 0.5, eps)
@@ -49,9 +52,8 @@ extern "C" pced_status pced_relevance(const float* ret_scores, int32_t ret_mode,
   if (((uintptr_t)ret_scores | (uintptr_t)r | (uintptr_t)rer_logits) & 3u)
     return fail(PCED_ERR_INVALID_ARG, "pced_relevance: pointers must be 4-byte aligned");
   if (num_sms() <= 0) return fail(PCED_ERR_NO_DEVICE, "pced_relevance: no CUDA device");
-  relevance_kernel<<<(n + REL_THREADS - 1) / REL_THREADS, REL_THREADS, 0, (cudaStream_t)stream>>>(
-      ret_scores, ret_mode, rer_logits, n, eps, r);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_pdl(relevance_kernel, dim3((n + REL_THREADS - 1) / REL_THREADS), REL_THREADS, 0,
+                                   (cudaStream_t)stream, ret_scores, ret_mode, rer_logits, n, eps, r);
   if (e != cudaSuccess) return cuda_status(e, "pced_relevance launch");
   return PCED_OK;
 }

@@ -32,7 +32,6 @@ struct StepLayout {
   float* sel_u;
   int32_t* sel_tok;
   float* lp;              // [S][V] log-probabilities of a dynamic-beta first step
-  void* ada;              // scratch of the beta kernel (counters zero between uses)
   float2* agg_part;       // MoE / PoE: per (query, expert, chunk) statistics
   float2* agg_best;       // MoE / PoE: per (query, chunk) best
   float* agg_best2;       // MoE / PoE: per (query, chunk) best at another token
@@ -78,7 +77,6 @@ static StepLayout step_layout(const pced_dims* dm, void* ws) {
   L.sel_u = c.take<float>((size_t)S);
   L.sel_tok = c.take<int32_t>((size_t)S);
   L.lp = c.take<float>((size_t)S * dm->V);
-  L.ada = c.take<char>(adacad_scratch_bytes(dm->B, dm->N, dm->V));
   L.agg_part = c.take<float2>((size_t)dm->B * dm->N * agg_chunks(dm->V));
   L.agg_best = c.take<float2>((size_t)dm->B * agg_chunks(dm->V));
   L.agg_best2 = c.take<float>((size_t)dm->B * agg_chunks(dm->V));
@@ -346,7 +344,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     // the JSD kernel also re-arms the LM head's tile counter for the fused pass
     if (e == cudaSuccess && dyn) {
       ranges.next("adacad_beta");
-      e = adacad_beta_launch(W.lp, dm.B, dm.N, dm.V, p->beta_out, W.ada, W.lm_tile_ctr, s);
+      e = adacad_beta_launch(W.lp, dm.B, dm.N, dm.V, p->beta_out, W.lm_tile_ctr, !timed, s);
       if (e == cudaSuccess) e = mark();
     }
     if (e != cudaSuccess) return cuda_status(e, "log-probability launches");
