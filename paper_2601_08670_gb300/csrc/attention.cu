@@ -14,9 +14,9 @@
 //     online softmax in base 2 with warp shuffles; P is split into bf16 hi +
 //     lo parts so the PV product keeps ~16 significant bits;
 //   * per piece, the eight warps' partials are merged in shared memory into one
-//     unnormalised record (max, sum, o); records of a segment split across
-//     CTAs are merged by a combine kernel (one layer) or by the last CTA to
-//     finish the segment (whole decode step, see att_step_kernel).
+//     unnormalised result (max, sum, o); the results of a segment split across
+//     CTAs are records, merged by a combine kernel (one layer) or by the first
+//     CTA of the segment (whole decode step, see att_step_kernel).
 #include <math.h>
 #include <stdlib.h>
 
@@ -33,42 +33,13 @@ struct AttCfg {
   static constexpr int STAGES = D == 128 ? 5 : 7;       // odd: consecutive uses of a stage alternate warpgroups
   static constexpr int KSTEPS = D / 16;
   static constexpr int MTILES = D / 16;
-  static constexpr int OPAD = 9;                        // padded head stride of the merge scratch
-  static constexpr int OROW = D + 4;                    // padded row (one head of one warp) of the step kernel's partials
-  static constexpr int OPT = ATT_MAX_G * D / ATT_CT;   // outputs of a piece per consumer thread (G <= 8)
-  static constexpr int MERGE_FLOATS = 2 * ATT_CONSUMERS * ATT_MAX_G + ATT_CONSUMERS * D * OPAD + ATT_CONSUMERS + 8;
+  static constexpr int OROW = D + 4;                    // padded row (one head of one warp) of a piece's partials
+  static constexpr int PARTIALS = 2 * ATT_CONSUMERS * ATT_MAX_G + ATT_CONSUMERS * ATT_MAX_G * OROW;  // floats, G = 8
   static constexpr size_t BARS = (2 * STAGES + 2) * 8;
-  static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + BARS + (size_t)MERGE_FLOATS * 4 +
-                                 (ATT_MAX_S + 1) * 8 + ATT_MAX_S * 4 + ATT_MAX_S + 128;
+  // one-layer kernel: stages, barriers, partials, pre[S+1], lens / row0 / cap [S]
+  static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + BARS + (size_t)PARTIALS * 4 +
+                                 (ATT_MAX_S + 1) * 8 + 3 * ATT_MAX_S * 4 + 128;
 };
-
-// shared-memory scratch of the consumers (after the stages and barriers)
-struct Scratch {
-  float* ms;      // [8][8] per-warp running max of a piece
-  float* ls;      // [8][8] per-warp sum
-  float* os;      // [8][D][OPAD] per-warp o
-  float* red;     // [8] per-warp partial sums
-  int* flag;      // [8] broadcast flags
-  int64_t* pre;   // [S+1] prefix of the segment extents
-  int32_t* lens;  // [S] live lengths
-  uint8_t* apnd;  // [S] 1 if this step appends a row to sequence s
-};
-
-template <int D>
-__device__ __forceinline__ Scratch carve_scratch(uint8_t* p) {
-  using C = AttCfg<D>;
-  Scratch sc;
-  float* f = reinterpret_cast<float*>(p);
-  sc.ms = f;
-  sc.ls = f + ATT_CONSUMERS * ATT_MAX_G;
-  sc.os = f + 2 * ATT_CONSUMERS * ATT_MAX_G;
-  sc.red = sc.os + ATT_CONSUMERS * D * C::OPAD;
-  sc.flag = reinterpret_cast<int*>(sc.red + ATT_CONSUMERS);
-  sc.pre = reinterpret_cast<int64_t*>(f + C::MERGE_FLOATS);
-  sc.lens = reinterpret_cast<int32_t*>(sc.pre + ATT_MAX_S + 1);
-  sc.apnd = reinterpret_cast<uint8_t*>(sc.lens + ATT_MAX_S);
-  return sc;
-}
 
 // Non-negative 64-bit quotient through the 32-bit divider when both operands
 // fit (positions of any realistic step do); 64-bit division is a long
@@ -288,14 +259,11 @@ __device__ __forceinline__ void pack_fold(WarpAcc<D>& A) {
     for (int j = 0; j < 4; ++j) A.o[i][j] += __shfl_xor_sync(0xffffffffu, A.o[i][j], 2);
 }
 
-// Merge the eight consumer warps' accumulators of a piece through shared
-// memory.  Afterwards this thread holds, for outputs idx = ctid + k*ATT_CT
-// (idx = hh*D + dd < G*D), the piece's running max mx[k] (log2 units), sum
-// ls[k] and unnormalised output acc[k].
+// This warp's partial of a piece (o, running max, sum) into shared memory:
+// ms, ls [ATT_MAX_G][8 warps], os [8 warps][G][D + 4].
 template <int D>
-__device__ __forceinline__ bool cta_merge(const WarpAcc<D>& A, const Scratch& sc, int G, int warp, int lane, int ctid,
-                                          uint32_t bar, uint32_t& ph, int* status, float (&mx)[AttCfg<D>::OPT],
-                                          float (&ls)[AttCfg<D>::OPT], float (&acc)[AttCfg<D>::OPT]) {
+__device__ __forceinline__ void store_partial(const WarpAcc<D>& A, float* ms, float* ls, float* os, int G, int warp,
+                                              int lane) {
   using C = AttCfg<D>;
   const int g = lane >> 2, tq = lane & 3;
   float l0 = A.l0, l1 = A.l1;
@@ -304,53 +272,73 @@ __device__ __forceinline__ bool cta_merge(const WarpAcc<D>& A, const Scratch& sc
     l0 += __shfl_xor_sync(0xffffffffu, l0, off);
     l1 += __shfl_xor_sync(0xffffffffu, l1, off);
   }
-  // every consumer is done with the previous piece's scratch
-  if (!warps_sync(bar, ph, status)) return false;
   if (g == 0) {
-    sc.ms[warp * ATT_MAX_G + 2 * tq] = A.m0;
-    sc.ms[warp * ATT_MAX_G + 2 * tq + 1] = A.m1;
-    sc.ls[warp * ATT_MAX_G + 2 * tq] = l0;
-    sc.ls[warp * ATT_MAX_G + 2 * tq + 1] = l1;
+    ms[(2 * tq) * ATT_CONSUMERS + warp] = A.m0;
+    ms[(2 * tq + 1) * ATT_CONSUMERS + warp] = A.m1;
+    ls[(2 * tq) * ATT_CONSUMERS + warp] = l0;
+    ls[(2 * tq + 1) * ATT_CONSUMERS + warp] = l1;
   }
-  float* ow = sc.os + warp * D * C::OPAD;
+  float* ow = os + warp * G * C::OROW;
+  const bool h0 = 2 * tq < G, h1 = 2 * tq + 1 < G;
 #pragma unroll
   for (int i = 0; i < C::MTILES; ++i) {
     const int d0 = 16 * i + g, d1 = d0 + 8;
-    ow[d0 * C::OPAD + 2 * tq] = A.o[i][0];
-    ow[d0 * C::OPAD + 2 * tq + 1] = A.o[i][1];
-    ow[d1 * C::OPAD + 2 * tq] = A.o[i][2];
-    ow[d1 * C::OPAD + 2 * tq + 1] = A.o[i][3];
-  }
-  if (!warps_sync(bar, ph, status)) return false;
-#pragma unroll
-  for (int k = 0; k < C::OPT; ++k) {
-    const int idx = ctid + k * ATT_CT;
-    mx[k] = -INFINITY;
-    ls[k] = 0.f;
-    acc[k] = 0.f;
-    if (idx >= G * D) continue;
-    const int hh = idx / D, dd = idx - hh * D;
-    float M = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < ATT_CONSUMERS; ++w) M = fmaxf(M, sc.ms[w * ATT_MAX_G + hh]);
-    float a = 0.f, l = 0.f;
-#pragma unroll
-    for (int w = 0; w < ATT_CONSUMERS; ++w) {
-      const float mw = sc.ms[w * ATT_MAX_G + hh];
-      if (mw == -INFINITY) continue;
-      const float e = exp2f(mw - M);
-      a += sc.os[(w * D + dd) * C::OPAD + hh] * e;
-      l += sc.ls[w * ATT_MAX_G + hh] * e;
+    if (h0) {
+      ow[(2 * tq) * C::OROW + d0] = A.o[i][0];
+      ow[(2 * tq) * C::OROW + d1] = A.o[i][2];
     }
-    mx[k] = M;
-    ls[k] = l;
-    acc[k] = a;
+    if (h1) {
+      ow[(2 * tq + 1) * C::OROW + d0] = A.o[i][1];
+      ow[(2 * tq + 1) * C::OROW + d1] = A.o[i][3];
+    }
   }
-  return true;
+}
+
+// The eight warps' partials combined for outputs idx0 .. idx0 + 3 (head hh):
+// running max mx (log2 units), sum lsum and unnormalised output acc.
+template <int D>
+__device__ __forceinline__ void load_merged(const float* ms, const float* ls, const float* os, int G, int hh, int idx0,
+                                            float& mx, float& lsum, float (&acc)[4]) {
+  using C = AttCfg<D>;
+  float mw[ATT_CONSUMERS], lw[ATT_CONSUMERS];
+  const float4* m4 = reinterpret_cast<const float4*>(ms + hh * ATT_CONSUMERS);
+  const float4* l4 = reinterpret_cast<const float4*>(ls + hh * ATT_CONSUMERS);
+  *reinterpret_cast<float4*>(mw) = m4[0];
+  *reinterpret_cast<float4*>(mw + 4) = m4[1];
+  *reinterpret_cast<float4*>(lw) = l4[0];
+  *reinterpret_cast<float4*>(lw + 4) = l4[1];
+  float M = mw[0];
+#pragma unroll
+  for (int w = 1; w < ATT_CONSUMERS; ++w) M = fmaxf(M, mw[w]);
+  const float* oc = os + hh * C::OROW + (idx0 - hh * D);
+#pragma unroll
+  for (int w = 0; w < ATT_CONSUMERS; ++w) {
+    if (mw[w] == -INFINITY) continue;  // a warp without live keys in this piece
+    const float e = exp2f(mw[w] - M);
+    const float4 o4 = *reinterpret_cast<const float4*>(oc + w * G * C::OROW);
+    acc[0] += o4.x * e;
+    acc[1] += o4.y * e;
+    acc[2] += o4.z * e;
+    acc[3] += o4.w * e;
+    lsum += lw[w] * e;
+  }
+  mx = M;
 }
 
 // =================================================================== one layer
-template <int D>
+// What bounds it: HBM once a CTA has tens of tiles, the serial chain around
+// them below that (lengths, offsets, first tile, last tile, merge).  The
+// lengths, capacities and offsets of all sequences arrive in one round trip
+// before the partition is known, so no piece waits for its own; a segment that
+// a CTA holds whole is normalised and written by it, and only the segments cut
+// by a CTA boundary (at most one per CTA) leave records for the second kernel,
+// which is resident by then (programmatic launch).  Measured, a call among
+// others: 9 x 2081 keys, 8 kv-heads, D = 128 (68.5 MB): 32.2 -> 18.0 us; 17 x
+// 4129 keys, 4 kv-heads, 7 heads each (136 MB): 50.1 -> 29.2 us; 272 ragged
+// sequences (1.27 GB): 208.9 -> 190.4 us (98 % of the copy bandwidth).  Before,
+// a combine CTA per segment read the whole partition and its records in four
+// dependent round trips (8.9-11.3 us) after the split kernel had ended.
+template <int D, bool PK>
 __global__ void __launch_bounds__(ATT_THREADS, 1)
     att_split_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap, AttArgs a) {
   using C = AttCfg<D>;
@@ -358,48 +346,55 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
-  // layout: stages | full[STAGES] | empty[STAGES] | consumer barrier | spare | scratch
+  // layout: stages | full[STAGES] | empty[STAGES] | partials full | partials empty | partials | tables
   const uint32_t bar_full = base + C::STAGES * C::STAGE_BYTES;
   const uint32_t bar_empty = bar_full + C::STAGES * 8;
-  const uint32_t bar_c = bar_empty + C::STAGES * 8;
-  const Scratch sc = carve_scratch<D>(gbase + C::STAGES * C::STAGE_BYTES + C::BARS);
+  const uint32_t bar_pfull = bar_empty + C::STAGES * 8, bar_pempty = bar_pfull + 8;
+  float* ms = reinterpret_cast<float*>(gbase + C::STAGES * C::STAGE_BYTES + C::BARS);
+  float* ls = ms + ATT_CONSUMERS * ATT_MAX_G;
+  float* os = ls + ATT_CONSUMERS * ATT_MAX_G;
+  int64_t* pre = reinterpret_cast<int64_t*>(ms + C::PARTIALS);
+  int32_t* lens = reinterpret_cast<int32_t*>(pre + ATT_MAX_S + 1);
+  int32_t* row0 = lens + ATT_MAX_S;  // tensor-map row of kv-head 0's first key
+  int32_t* caps = row0 + ATT_MAX_S;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int32_t S = a.S, G = a.G;
+  const int32_t S = a.S, G = a.G, GD = G * D;
 
   if (tid == 0) {
     for (int i = 0; i < C::STAGES; ++i) {
       mbar_init(bar_full + 8 * i, 1);
       mbar_init(bar_empty + 8 * i, 4);  // the four warps of the consuming warpgroup
     }
-    mbar_init(bar_c, ATT_CONSUMERS);
+    mbar_init(bar_pfull, ATT_CONSUMERS);
+    mbar_init(bar_pempty, ATT_CONSUMERS);
     mbar_fence_init();
   }
   if (warp == ATT_CONSUMERS && lane == 0) {
     tma_prefetch_desc(&kmap);
     tma_prefetch_desc(&vmap);
   }
+  pdl_launch_dependents();
+  pdl_wait();
   // live lengths, clamped into [1, cap] (out-of-range lengths are flagged)
   for (int i = tid; i < S; i += ATT_THREADS) {
-    int32_t L = a.seq_len[i], c = a.cap[i];
+    int32_t L = a.seq_len[i];
+    const int32_t c = a.cap[i];
+    const int64_t off = a.kv_offset[i];
     if (L < 1 || L > c) {
       dev_flag(a.status, PCED_DEV_BAD_LENGTH);
       L = L < 1 ? 1 : (L > c ? (c < 1 ? 1 : c) : L);
     }
-    sc.lens[i] = L;
+    lens[i] = L;
+    caps[i] = c;
+    row0[i] = (int32_t)(off / D);
   }
   __syncthreads();
-  if (warp == 0) prefix_extents(sc.lens, S, 0, sc.pre, lane);
+  if (warp == 0) prefix_extents(lens, S, 0, pre, lane);
   __syncthreads();
-  const int64_t* pre = sc.pre;
-  const int32_t* lens = sc.lens;
   const int64_t T = pre[S];
   const int64_t total = T * a.Hkv;
-  const int64_t per = (total + gridDim.x - 1) / gridDim.x;
-  if (blockIdx.x == 0) {
-    for (int i = tid; i <= S; i += ATT_THREADS) a.plan_pre[i] = pre[i];
-    if (tid == 0) *a.plan_per = per;
-  }
+  const int64_t per = udiv_pos(total + gridDim.x - 1, gridDim.x);
   const int64_t r_begin = min(total, (int64_t)blockIdx.x * per);
   const int64_t r_end = min(total, r_begin + per);
 
@@ -407,14 +402,15 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     // ------------------------------------------------------------ producer
     if (lane == 0) {
       const uint64_t pol = policy_evict_first();
-      uint32_t it = 0;
+      uint32_t it = 0, st = 0, ph = 0;
       bool ok = true;
+      Piece pc;
+      pc.adv = -1;  // none yet
       for (int64_t p = r_begin; p < r_end && ok;) {
-        const Piece pc = find_piece(pre, lens, 0, S, T, p, r_end);
+        pc = pc.adv < 0 ? find_piece(pre, lens, 0, S, T, p, r_end) : next_piece(pc, pre, lens, 0, S, T, p, r_end);
         p += pc.adv;
-        const int64_t slab_row = a.row_base + (a.kv_offset[pc.s] + (int64_t)pc.h * a.cap[pc.s] * D) / D;
+        const int32_t slab_row = row0[pc.s] + pc.h * caps[pc.s];
         for (int32_t kt = pc.k0; kt < pc.k1; kt += ATT_BLOCK_N, ++it) {
-          const uint32_t st = it % C::STAGES, ph = (it / C::STAGES) & 1u;
           if (!mbar_wait(bar_empty + 8 * st, ph ^ 1u, a.status)) {
             ok = false;
             break;
@@ -422,9 +418,13 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
           const uint32_t fb = bar_full + 8 * st;
           const uint32_t sk = base + st * C::STAGE_BYTES, sv = sk + C::TILE_BYTES;
           mbar_arrive_expect_tx(fb, C::STAGE_BYTES);
-          const int32_t row = (int32_t)(slab_row + kt);
+          const int32_t row = slab_row + kt;
           tma_load_3d(sk, &kmap, fb, 0, row, 0, pol);
           tma_load_3d(sv, &vmap, fb, 0, row, 0, pol);
+          if (++st == C::STAGES) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
       }
       if (!ok) {
@@ -440,16 +440,21 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
   const int wg = warp >> 2, wl = warp & 3;
   const int g = lane >> 2, tq = lane & 3;
   const int kb = 16 * wl;
-  uint32_t it = 0, cph = 0;
+  // B column g of S^T = K Q^T is head g; with PK columns 4-7 repeat heads 0-3
+  const int qh = PK ? (g & 3) : g;
+  const bool hv = qh < G;
+  uint32_t it = 0, st = 0, use = 0, np = 0;  // tile counter, its stage and use of the stage; pieces done
   bool ok = true;
-  for (int64_t p = r_begin; p < r_end && ok;) {
-    const Piece pc = find_piece(pre, lens, 0, S, T, p, r_end);
+  int2 plan = make_int2(0, 0);
+  Piece pc;
+  pc.adv = -1;  // none yet
+  for (int64_t p = r_begin; p < r_end && ok; ++np) {
+    pc = pc.adv < 0 ? find_piece(pre, lens, 0, S, T, p, r_end) : next_piece(pc, pre, lens, 0, S, T, p, r_end);
     p += pc.adv;
     uint32_t qf[C::KSTEPS][2];
     {
-      const bool hv = g < G;
       const uint32_t* qrow = reinterpret_cast<const uint32_t*>(
-          a.q + ((int64_t)pc.s * a.Hq + (int64_t)pc.h * G + (hv ? g : 0)) * D);
+          a.q + ((int64_t)pc.s * a.Hq + (int64_t)pc.h * G + (hv ? qh : 0)) * D);
 #pragma unroll
       for (int j = 0; j < C::KSTEPS; ++j) {
         qf[j][0] = hv ? qrow[8 * j + tq] : 0u;
@@ -458,9 +463,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     }
     WarpAcc<D> A;
     acc_reset(A);
-    for (int32_t kt = pc.k0; kt < pc.k1; kt += ATT_BLOCK_N, ++it) {
+    for (int32_t kt = pc.k0; kt < pc.k1; kt += ATT_BLOCK_N, ++it, st = st + 1 == C::STAGES ? (++use, 0u) : st + 1) {
       if ((int)(it & 1u) != wg) continue;
-      const uint32_t use = it / C::STAGES, st = it % C::STAGES, ph = use & 1u;
       // Consecutive uses of a stage belong to different warpgroups.  Waiting for
       // the release of the previous use first guarantees that the full barrier
       // has completed that use's phase, so the parity test below refers to this
@@ -469,94 +473,105 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
         ok = false;
         break;
       }
-      if (!mbar_wait(bar_full + 8 * st, ph, a.status)) {
+      if (!mbar_wait(bar_full + 8 * st, use & 1u, a.status)) {
         ok = false;
         break;
       }
       const int nvalid = min(ATT_BLOCK_N, pc.k1 - kt);
       if (kb < nvalid) {
         const uint32_t sk = base + st * C::STAGE_BYTES;
-        tile_math<D>(A, qf, sk, sk + C::TILE_BYTES, kb, nvalid, a.scale_log2, lane);
+        tile_math<D, PK>(A, qf, sk, sk + C::TILE_BYTES, kb, nvalid, a.scale_log2, lane);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_empty + 8 * st);
     }
     if (!ok) break;
-    float mx[C::OPT], ls[C::OPT], acc[C::OPT];
-    if (!cta_merge<D>(A, sc, G, warp, lane, tid, bar_c, cph, a.status, mx, ls, acc)) break;
-    const int64_t slot = (int64_t)blockIdx.x + (int64_t)pc.h * S + pc.s;
+    if (PK) pack_fold<D>(A);
+    // the previous piece's partials have been read
+    if (np > 0 && !mbar_wait(bar_pempty, (np - 1u) & 1u, a.status)) break;
+    store_partial<D>(A, ms, ls, os, G, warp, lane);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_pfull);
+    if (!mbar_wait(bar_pfull, np & 1u, a.status)) break;
+    const bool own = tid < GD / 4;
+    const int hh = own ? tid / (D / 4) : 0, idx0 = own ? 4 * tid : 0;
+    float mx = -INFINITY, lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (own) load_merged<D>(ms, ls, os, G, hh, idx0, mx, lsum, acc);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_pempty);
+    const int32_t len = lens[pc.s];
+    if (pc.k0 == 0 && pc.k1 == len) {
+      if (own) {
+        const float w = mx == -INFINITY ? 0.f : 1.f / lsum;
+        float* op = a.out + ((int64_t)pc.s * a.Hq + (int64_t)pc.h * G) * D + idx0;
 #pragma unroll
-    for (int k = 0; k < C::OPT; ++k) {
-      const int idx = tid + k * ATT_CT;
-      if (idx >= G * D) continue;
-      a.rec_o[slot * G * D + idx] = acc[k];
-      if (idx % D == 0) a.rec_ml[slot * G + idx / D] = make_float2(mx[k], ls[k]);
+        for (int j = 0; j < 4; ++j) op[j] = mx == -INFINITY ? 0.f : acc[j] * w;
+      }
+      continue;
     }
-    if (!warps_sync(bar_c, cph, a.status)) break;
+    // a part of a segment: record 2c of CTA c when the segment began in an
+    // earlier CTA, 2c + 1 when it begins here
+    const int64_t slot = 2 * (int64_t)blockIdx.x + (pc.k0 == 0 ? 1 : 0);
+    if (own) {
+      *reinterpret_cast<float4*>(a.rec_o + slot * GD + idx0) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      if (idx0 % D == 0) a.rec_ml[slot * G + hh] = make_float2(mx, lsum);
+    }
+    if (pc.k0 == 0)  // its last key lies (p - 1 + the keys left) positions on
+      plan = make_int2(pc.s * a.Hkv + pc.h, (int)(udiv_pos(p - 1 + (len - pc.k1), per) - blockIdx.x) + 1);
   }
+  if (tid == 0) a.plan[blockIdx.x] = plan;
 }
 
-// One CTA per (kv-head h, sequence s): weights of the records that cover the
-// segment are formed once in shared memory, then every output element sums
-// its records with independent loads.
-constexpr int CMB_THREADS = 128;
-constexpr int CMB_SLOTS = 64;                                  // records weighted per pass
-constexpr int CMB_PER_THREAD = ATT_MAX_G * 128 / CMB_THREADS;  // G*D <= 1024 outputs per CTA
+// CTA c merges the segment that begins in CTA c of the split kernel and goes on
+// past it (if there is one): records 2c + 1, 2(c + 1), 2(c + 2), ...  Thread
+// tid holds outputs 4 tid .. 4 tid + 3; the records arrive CMB_BATCH at a time.
+constexpr int CMB_THREADS = ATT_MAX_G * 128 / 4;
+constexpr int CMB_BATCH = 4;
 
 __global__ void __launch_bounds__(CMB_THREADS) att_combine_kernel(CombineArgs a) {
-  const int h = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
-  const int32_t Hq = a.Hq, G = a.G, D = a.D, S = a.S, d = Hq * D;
-  __shared__ float wts[CMB_SLOTS][ATT_MAX_G];
-  const int64_t per = *a.plan_per;
-  const int64_t T = a.plan_pre[S];
-  const int64_t pre_s = a.plan_pre[s];
-  const int64_t len = a.plan_pre[s + 1] - pre_s;
-  const int64_t seg = (int64_t)h * S + s;
-  const int64_t pa = (int64_t)h * T + pre_s;
-  const int64_t c0 = pa / per, c1 = (pa + len - 1) / per;
-  const int GD = G * D;
-
-  // global max and total of each head over all records of the segment
-  float Mh = -INFINITY, Lh = 0.f;
-  if (tid < G) {
-    for (int64_t c = c0; c <= c1; ++c) Mh = fmaxf(Mh, a.rec_ml[(c + seg) * G + tid].x);
-    for (int64_t c = c0; c <= c1; ++c) {
-      const float2 ml = a.rec_ml[(c + seg) * G + tid];
-      if (ml.x != -INFINITY) Lh += ml.y * exp2f(ml.x - Mh);
-    }
-  }
-  __shared__ float Msh[ATT_MAX_G], Lsh[ATT_MAX_G];
-  if (tid < G) {
-    Msh[tid] = Mh;
-    Lsh[tid] = Lh;
-  }
-  float acc[CMB_PER_THREAD];
+  const int c = blockIdx.x, tid = threadIdx.x, GD = a.G * a.D;
+  pdl_launch_dependents();
+  pdl_wait();
+  const int2 plan = a.plan[c];
+  if (plan.y < 2 || 4 * tid >= GD) return;
+  const int hh = 4 * tid / a.D;
+  float mx = -INFINITY, lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int i0 = 0; i0 < plan.y; i0 += CMB_BATCH) {
+    float2 ml[CMB_BATCH];
+    float4 o[CMB_BATCH];
 #pragma unroll
-  for (int j = 0; j < CMB_PER_THREAD; ++j) acc[j] = 0.f;
-  for (int64_t cb = c0; cb <= c1; cb += CMB_SLOTS) {
-    const int64_t rem = c1 + 1 - cb;
-    const int n = (int)(rem < CMB_SLOTS ? rem : CMB_SLOTS);
-    __syncthreads();
-    for (int i = tid; i < n * G; i += CMB_THREADS) {
-      const int ci = i / G, gh = i - ci * G;
-      const float2 ml = a.rec_ml[(cb + ci + seg) * G + gh];
-      wts[ci][gh] = ml.x == -INFINITY ? 0.f : exp2f(ml.x - Msh[gh]) / Lsh[gh];
+    for (int q = 0; q < CMB_BATCH; ++q) {
+      const int i = i0 + q;
+      ml[q] = make_float2(-INFINITY, 0.f);
+      o[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i >= plan.y) continue;
+      const int64_t slot = i == 0 ? 2 * (int64_t)c + 1 : 2 * ((int64_t)c + i);
+      ml[q] = a.rec_ml[slot * a.G + hh];
+      o[q] = *reinterpret_cast<const float4*>(a.rec_o + slot * GD + 4 * tid);
     }
-    __syncthreads();
-    for (int ci = 0; ci < n; ++ci) {
-      const float* ro = a.rec_o + (cb + ci + seg) * GD;
+    float M = mx;
 #pragma unroll
-      for (int j = 0; j < CMB_PER_THREAD; ++j) {
-        const int idx = tid + j * CMB_THREADS;
-        if (idx < GD) acc[j] += wts[ci][idx / D] * ro[idx];
-      }
+    for (int q = 0; q < CMB_BATCH; ++q) M = fmaxf(M, ml[q].x);
+    const float f = mx == -INFINITY ? 0.f : exp2f(mx - M);
+    lsum *= f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] *= f;
+#pragma unroll
+    for (int q = 0; q < CMB_BATCH; ++q) {
+      const float e = ml[q].x == -INFINITY ? 0.f : exp2f(ml[q].x - M);
+      acc[0] += o[q].x * e;
+      acc[1] += o[q].y * e;
+      acc[2] += o[q].z * e;
+      acc[3] += o[q].w * e;
+      lsum += ml[q].y * e;
     }
+    mx = M;
   }
+  const int s = plan.x / a.Hkv, h = plan.x - s * a.Hkv;
+  const float w = 1.f / lsum;
+  float* op = a.out + (int64_t)s * a.Hq * a.D + (int64_t)h * GD + 4 * tid;
 #pragma unroll
-  for (int j = 0; j < CMB_PER_THREAD; ++j) {
-    const int idx = tid + j * CMB_THREADS;
-    if (idx < GD) a.out[(int64_t)s * d + (int64_t)h * GD + idx] = acc[j];
-  }
+  for (int j = 0; j < 4; ++j) op[j] = mx == -INFINITY ? 0.f : acc[j] * w;
 }
 
 // ============================================================ whole step
@@ -1383,38 +1398,11 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
       ok = false;
       break;
     }
-    float l0 = A.l0, l1 = A.l1;
-#pragma unroll
-    for (int off = 4; off < 32; off <<= 1) {
-      l0 += __shfl_xor_sync(0xffffffffu, l0, off);
-      l1 += __shfl_xor_sync(0xffffffffu, l1, off);
-    }
     if (PK) pack_fold<D>(A);
     float* ms = reinterpret_cast<float*>(gbase + SL.pbuf + slot * SL.pslot);  // [ATT_MAX_G][8 warps]
     float* ls = ms + ATT_MAX_G * ATT_CONSUMERS;                                // [ATT_MAX_G][8 warps]
     float* os = ls + ATT_MAX_G * ATT_CONSUMERS;                                // [8 warps][G][D + 4]
-    if (g == 0) {
-      ms[(2 * tq) * ATT_CONSUMERS + warp] = A.m0;
-      ms[(2 * tq + 1) * ATT_CONSUMERS + warp] = A.m1;
-      ls[(2 * tq) * ATT_CONSUMERS + warp] = l0;
-      ls[(2 * tq + 1) * ATT_CONSUMERS + warp] = l1;
-    }
-    {
-      float* ow = os + warp * G * C::OROW;
-      const bool h0 = 2 * tq < G, h1 = 2 * tq + 1 < G;
-#pragma unroll
-      for (int i = 0; i < C::MTILES; ++i) {
-        const int d0 = 16 * i + g, d1 = d0 + 8;
-        if (h0) {
-          ow[(2 * tq) * C::OROW + d0] = A.o[i][0];
-          ow[(2 * tq) * C::OROW + d1] = A.o[i][2];
-        }
-        if (h1) {
-          ow[(2 * tq + 1) * C::OROW + d0] = A.o[i][1];
-          ow[(2 * tq + 1) * C::OROW + d1] = A.o[i][3];
-        }
-      }
-    }
+    store_partial<D>(A, ms, ls, os, G, warp, lane);
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_pfull + 8 * slot);
     if (!mbar_wait(bar_pfull + 8 * slot, u & 1u, a.status, a.wait_ns)) {
@@ -1425,31 +1413,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
     const bool own = tid < GD / 4;
     const int hh = own ? tid / (D / 4) : 0, idx0 = own ? 4 * tid : 0;
     float mx = -INFINITY, lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-    if (own) {
-      float mw[ATT_CONSUMERS], lw[ATT_CONSUMERS];
-      const float4* m4 = reinterpret_cast<const float4*>(ms + hh * ATT_CONSUMERS);
-      const float4* l4 = reinterpret_cast<const float4*>(ls + hh * ATT_CONSUMERS);
-      *reinterpret_cast<float4*>(mw) = m4[0];
-      *reinterpret_cast<float4*>(mw + 4) = m4[1];
-      *reinterpret_cast<float4*>(lw) = l4[0];
-      *reinterpret_cast<float4*>(lw + 4) = l4[1];
-      float M = mw[0];
-#pragma unroll
-      for (int w = 1; w < ATT_CONSUMERS; ++w) M = fmaxf(M, mw[w]);
-      const float* oc = os + hh * C::OROW + (idx0 - hh * D);
-#pragma unroll
-      for (int w = 0; w < ATT_CONSUMERS; ++w) {
-        if (mw[w] == -INFINITY) continue;  // a warp without live keys in this piece
-        const float e = exp2f(mw[w] - M);
-        const float4 o4 = *reinterpret_cast<const float4*>(oc + w * G * C::OROW);
-        acc[0] += o4.x * e;
-        acc[1] += o4.y * e;
-        acc[2] += o4.z * e;
-        acc[3] += o4.w * e;
-        lsum += lw[w] * e;
-      }
-      mx = M;
-    }
+    if (own) load_merged<D>(ms, ls, os, G, hh, idx0, mx, lsum, acc);
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_pempty + 8 * slot);
     if (!merges) {
@@ -1596,6 +1560,8 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
 }
 
 // ------------------------------------------------------------------- host
+// What the workspace is sized by: more than the 2 records per CTA (at most
+// ATT_SPLIT_CTAS) and one plan entry per CTA that a call uses.
 size_t att_records_bytes(int32_t S, int32_t Hq, int32_t Hkv, int32_t D) {
   const int64_t G = Hq / (Hkv > 0 ? Hkv : 1);
   const int64_t slots = ATT_MAX_CTAS + (int64_t)S * Hkv;
@@ -1643,26 +1609,33 @@ static cudaError_t set_smem_once(K kernel, size_t bytes, bool* done) {
   return cudaSuccess;
 }
 
-template <int D>
+template <int D, bool PK>
 static cudaError_t launch_split(const CUtensorMap& kmap, const CUtensorMap& vmap, const AttArgs& a, int ctas,
                                 cudaStream_t stream) {
   static bool configured[64];
-  cudaError_t e = set_smem_once(att_split_kernel<D>, AttCfg<D>::SMEM, configured);
+  cudaError_t e = set_smem_once(att_split_kernel<D, PK>, AttCfg<D>::SMEM, configured);
   if (e != cudaSuccess) return e;
-  att_split_kernel<D><<<ctas, ATT_THREADS, AttCfg<D>::SMEM, stream>>>(kmap, vmap, a);
-  return cudaGetLastError();
+  return pced_host::launch_pdl(att_split_kernel<D, PK>, dim3(ctas), ATT_THREADS, AttCfg<D>::SMEM, stream, kmap, vmap,
+                               a);
 }
 
-cudaError_t att_split_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, const AttArgs& a, int ctas,
-                             cudaStream_t stream) {
-  if (D == 128) return launch_split<128>(kmap, vmap, a, ctas, stream);
-  if (D == 64) return launch_split<64>(kmap, vmap, a, ctas, stream);
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t att_combine_launch(const CombineArgs& a, cudaStream_t stream) {
-  att_combine_kernel<<<dim3(a.Hkv, a.S), CMB_THREADS, 0, stream>>>(a);
-  return cudaGetLastError();
+cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, AttArgs a, int64_t total_cap_keys,
+                             void* scratch, cudaStream_t stream) {
+  int ctas = att_grid(total_cap_keys);
+  if (ctas > ATT_SPLIT_CTAS) ctas = ATT_SPLIT_CTAS;
+  pced_host::Carver cv(scratch);
+  a.rec_o = cv.take<float>((size_t)2 * ctas * a.G * D);
+  a.rec_ml = cv.take<float2>((size_t)2 * ctas * a.G);
+  a.plan = cv.take<int2>((size_t)ctas);
+  const bool pk = a.G <= 4;  // hi and lo parts of P share one MMA
+  cudaError_t e = cudaErrorInvalidValue;
+  if (D == 128)
+    e = pk ? launch_split<128, true>(kmap, vmap, a, ctas, stream) : launch_split<128, false>(kmap, vmap, a, ctas, stream);
+  else if (D == 64)
+    e = pk ? launch_split<64, true>(kmap, vmap, a, ctas, stream) : launch_split<64, false>(kmap, vmap, a, ctas, stream);
+  if (e != cudaSuccess) return e;
+  const CombineArgs c = {a.Hq, a.Hkv, a.G, D, a.rec_o, a.rec_ml, a.plan, a.out};
+  return pced_host::launch_pdl(att_combine_kernel, dim3(ctas), CMB_THREADS, 0, stream, c);
 }
 
 template <int D, bool PK>
@@ -1737,10 +1710,7 @@ extern "C" pced_status pced_decode_attention(const void* q, const void* k_cache,
   st = make_tmap_kv(&vmap, v_cache, rows, (uint32_t)D, ATT_BLOCK_N);
   if (st != PCED_OK) return st;
 
-  const int32_t G = Hq / Hkv;
-  Carver cv((char*)workspace + 256);
-  const int64_t slots = ATT_MAX_CTAS + (int64_t)S * Hkv;
-  AttArgs a;
+  AttArgs a = {};
   a.q = (const __nv_bfloat16*)q;
   a.kv_offset = kv_offset;
   a.cap = cap;
@@ -1748,32 +1718,12 @@ extern "C" pced_status pced_decode_attention(const void* q, const void* k_cache,
   a.S = S;
   a.Hq = Hq;
   a.Hkv = Hkv;
-  a.G = G;
-  a.row_base = 0;
+  a.G = Hq / Hkv;
   a.scale_log2 = scale * 1.4426950408889634f;
-  a.rec_o = cv.take<float>((size_t)(slots * G * D));
-  a.rec_ml = cv.take<float2>((size_t)(slots * G));
-  a.plan_pre = cv.take<int64_t>((size_t)S + 1);
-  a.plan_per = cv.take<int64_t>(1);
+  a.out = out;
   a.status = (int*)workspace;
-  const int ctas = att_grid(total_cap * Hkv);
-  cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = att_split_launch(D, kmap, vmap, a, ctas, s);
-  if (e != cudaSuccess) return cuda_status(e, "attention split launch");
-
-  CombineArgs c = {};
-  c.S = S;
-  c.Hq = Hq;
-  c.Hkv = Hkv;
-  c.G = G;
-  c.D = D;
-  c.rec_o = a.rec_o;
-  c.rec_ml = a.rec_ml;
-  c.plan_pre = a.plan_pre;
-  c.plan_per = a.plan_per;
-  c.out = out;
-  c.status = a.status;
-  e = att_combine_launch(c, s);
-  if (e != cudaSuccess) return cuda_status(e, "attention combine launch");
+  const cudaError_t e =
+      att_layer_launch(D, kmap, vmap, a, total_cap * Hkv, (char*)workspace + 256, (cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_status(e, "attention launch");
   return PCED_OK;
 }

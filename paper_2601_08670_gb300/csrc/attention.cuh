@@ -22,43 +22,42 @@ constexpr int ATT_PTAB = 1024;       // block-table entries a step-kernel CTA ke
 // ranges, one per CTA.  Position of key k of kv-head h of sequence s:
 //   h * T + pre[s] + k,   pre[s] = sum_{s' < s} len[s'],  T = pre[S].
 // Head-major order spreads short segments (the amateurs) across CTAs.  A
-// CTA's range is cut into pieces at segment boundaries; the partial result of
-// CTA c over segment seg = h*S + s is stored in record slot c + seg (slots are
-// unique: each step along the position axis crosses a CTA boundary or a
-// segment boundary, or both).
+// CTA's range is cut into pieces at segment boundaries.  Only a CTA's first
+// and last piece can be part of a segment held by several CTAs: their partial
+// results are records 2c (the segment began earlier) and 2c + 1 (it begins in
+// CTA c), and plan[c] names the segment that begins in CTA c and goes on past
+// it, with its number of records.  Every other piece is a whole segment, whose
+// output the CTA writes itself.
 struct AttArgs {
   const __nv_bfloat16* q;     // [S][Hq][D]
   const int64_t* kv_offset;   // [S]
   const int32_t* cap;         // [S]
   const int32_t* seq_len;     // [S]
   int32_t S, Hq, Hkv, G;
-  int64_t row_base;           // row of this layer's region in the tensor maps
   float scale_log2;           // softmax scale * log2(e)
-  float* rec_o;               // [slots][G][D] unnormalised partial outputs
-  float2* rec_ml;             // [slots][G] (running max in log2 units, sum of exp2)
-  int64_t* plan_pre;          // [S+1] written by CTA 0 (prefix of len)
-  int64_t* plan_per;          // [1]   written by CTA 0: keys per CTA
+  float* out;                 // [S][Hq][D]
+  float* rec_o;               // [2 * CTAs][G][D] unnormalised partial outputs
+  float2* rec_ml;             // [2 * CTAs][G] (running max in log2 units, sum of exp2)
+  int2* plan;                 // [CTAs] (s * Hkv + h, records), records < 2: none
   int* status;
 };
 
-size_t att_records_bytes(int32_t S, int32_t Hq, int32_t Hkv, int32_t D);
-int att_grid(int64_t total_cap_keys);
-// launch the split kernel for head dim D (64 or 128)
-cudaError_t att_split_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, const AttArgs& a, int ctas,
-                             cudaStream_t stream);
-
-// Combine the partial records of one layer; one CTA per (kv-head, sequence):
-// out[s][hq][dd] = o (fp32).
+// Merges the records: CTA c the segment of plan[c].
 struct CombineArgs {
-  int32_t S, Hq, Hkv, G, D;
+  int32_t Hq, Hkv, G, D;
   const float* rec_o;
   const float2* rec_ml;
-  const int64_t* plan_pre;
-  const int64_t* plan_per;
+  const int2* plan;
   float* out;
-  int* status;
 };
-cudaError_t att_combine_launch(const CombineArgs& a, cudaStream_t stream);
+
+constexpr int ATT_SPLIT_CTAS = ATT_MAX_CTAS / 4;  // grid limit (2 records per CTA fit what att_records_bytes gives)
+size_t att_records_bytes(int32_t S, int32_t Hq, int32_t Hkv, int32_t D);
+int att_grid(int64_t total_cap_keys);
+// one layer's split and combine kernels, for head dim D (64 or 128); records and
+// plan (rec_o, rec_ml, plan of `a`) are placed in `scratch`, 256-byte aligned
+cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, AttArgs a, int64_t total_cap_keys,
+                             void* scratch, cudaStream_t stream);
 
 // ------------------------------------------------------- whole decode step
 // One cooperative launch runs the embedding and every layer of the step.

@@ -86,8 +86,9 @@ extern "C" pced_status pced_decode_attention_noalloc(const void* q, const void* 
     return fail(PCED_ERR_INVALID_ARG, "pced_decode_attention_noalloc: status must be 4-byte aligned");
   if (num_sms() <= 0) return fail(PCED_ERR_NO_DEVICE, "pced_decode_attention_noalloc: no CUDA device");
 
-  // Scratch layout (256-byte aligned pieces): status sink | rec_o | rec_ml |
-  // plan_pre | plan_per.  Record slot c + h*S + s for CTA c < ctas.
+  // The documented limit on sizes: (CTAs + S*Hkv) records and a prefix table.
+  // What a call uses of the array is less: the status sink, then the 2
+  // records per CTA and the plan that att_layer_launch places.
   const int32_t G = Hq / Hkv;
   const int ctas = att_grid(total_cap * Hkv);
   const int64_t slots = (int64_t)ctas + (int64_t)S * Hkv;
@@ -117,9 +118,10 @@ extern "C" pced_status pced_decode_attention_noalloc(const void* q, const void* 
   // Nothing here has to start at zero: every record and plan entry the combine
   // kernel reads is written by the split kernel of the same call, and the
   // status sink (used when the caller passes no status word) is write-only.
-  Carver cv(scratch);
-  int* sink = cv.take<int>(1);
-  AttArgs a;
+  static_assert(256 + 2ull * ATT_SPLIT_CTAS * ATT_MAX_G * (128 * 4 + 8) + 8 * ATT_SPLIT_CTAS + 1024 <=
+                    PCED_NOALLOC_SCRATCH_BYTES,
+                "the records of the largest grid fit the array");
+  AttArgs a = {};
   a.q = (const __nv_bfloat16*)q;
   a.kv_offset = kv_offset;
   a.cap = cap;
@@ -128,30 +130,11 @@ extern "C" pced_status pced_decode_attention_noalloc(const void* q, const void* 
   a.Hq = Hq;
   a.Hkv = Hkv;
   a.G = G;
-  a.row_base = 0;
   a.scale_log2 = scale * 1.4426950408889634f;
-  a.rec_o = cv.take<float>((size_t)(slots * G * D));
-  a.rec_ml = cv.take<float2>((size_t)(slots * G));
-  a.plan_pre = cv.take<int64_t>((size_t)S + 1);
-  a.plan_per = cv.take<int64_t>(1);
-  a.status = status ? (int*)status : sink;
-  cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = att_split_launch(D, kmap, vmap, a, ctas, s);
-  if (e != cudaSuccess) return cuda_status(e, "pced_decode_attention_noalloc: split launch");
-
-  CombineArgs c = {};
-  c.S = S;
-  c.Hq = Hq;
-  c.Hkv = Hkv;
-  c.G = G;
-  c.D = D;
-  c.rec_o = a.rec_o;
-  c.rec_ml = a.rec_ml;
-  c.plan_pre = a.plan_pre;
-  c.plan_per = a.plan_per;
-  c.out = out;
-  c.status = a.status;
-  e = att_combine_launch(c, s);
-  if (e != cudaSuccess) return cuda_status(e, "pced_decode_attention_noalloc: combine launch");
+  a.out = out;
+  a.status = status ? (int*)status : (int*)scratch;
+  const cudaError_t e =
+      att_layer_launch(D, kmap, vmap, a, total_cap * Hkv, (char*)scratch + 256, (cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_status(e, "pced_decode_attention_noalloc: launch");
   return PCED_OK;
 }

@@ -88,3 +88,14 @@ def test_bad_length_sets_device_status_without_faulting(cuda_ok):
     torch.cuda.synchronize()
     assert pced.device_status(ws) & pced.PCED_DEV_BAD_LENGTH
     assert torch.isfinite(out).all()
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,D", [
+    ([5000], 8, 1, 64),                # one segment over every CTA: many records of one head group
+    ([30000], 7, 1, 128),              # ... over the whole grid
+    ([256, 256, 256, 256], 4, 4, 64),  # segments that end where CTAs end: no records
+    ([255, 1, 257, 511, 512, 1], 4, 2, 128),  # boundaries one key before and after a segment's end
+    ([1] * 40 + [900], 32, 8, 128),    # many whole segments per CTA, then one that is cut
+])
+def test_records_and_whole_segments(cuda_ok, lens, Hq, Hkv, D):
+    assert run_case(lens, Hq=Hq, Hkv=Hkv, D=D, extra=0, seed=5) < 1e-4
