@@ -23,7 +23,7 @@ ROOT = os.path.dirname(HERE)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", os.path.join(ROOT, "include")]
-SOURCES = ["attention.cu", "attention_noalloc.cu", "lm_head.cu", "select.cu", "adacad.cu", "aggregate.cu", "relevance.cu",
+SOURCES = ["attention.cu", "attention_noalloc.cu", "lm_head.cu", "lm_head_pair.cu", "select.cu", "adacad.cu", "aggregate.cu", "relevance.cu",
            "step.cu", "partition.cu", "host.cu"]
 
 

@@ -5,10 +5,11 @@
 // Swap-AB skinny GEMM: Z^T[V x S] = W[V x d] * H^T[d x S].  The vocabulary is
 // the UMMA M dimension (128-row tiles), the S hidden rows are the N dimension,
 // so the bf16 unembedding matrix streams from HBM exactly once per step while
-// the tiny H operand is re-read from L2.  Persistent CTAs, one per SM:
+// the tiny H operand is re-read from L2 (from LM_PAIR_MIN_S rows on by pairs of
+// CTAs, lm_head_pair.cu).  Persistent CTAs, one per SM:
 //   warp 0  TMA producer (W tile 128x64 + H slab S_pad x 64 per stage, 128B swizzle)
 //   warp 1  TMEM allocator and single-thread tcgen05.mma issuer (fp32 accumulators
-//           in TMEM, double-buffered when 2*S_pad <= 512 columns)
+//           in TMEM, double-buffered)
 //   warps 2-9 epilogue: tcgen05.ld of the 128 x S accumulator (warp w reads TMEM lane
 //           quarter w % 4; warps 2-5 take the first half of the columns, 6-9 the rest);
 //           per column the tile's (max, sum exp) for the log-softmax and, for each
@@ -21,228 +22,131 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include "lm_epilogue.cuh"
 #include "lm_head.cuh"
 #include "select_key.cuh"
 
 namespace pced {
 
-constexpr int LM_A_BYTES = LM_TILE_V * LM_TILE_K * 2;  // 16 KB
-constexpr size_t LM_SMEM_BUDGET = 227 * 1024;
+constexpr int LM_PAIR_HSTAGES = 4;  // most stages of a pair's H ring
 
 bool lm_geometry(int32_t S, int32_t d, int32_t V, LmGeom* g) {
   if (S < 1 || S > LM_MAX_S || d < LM_TILE_K || d % LM_TILE_K != 0 || V < 1) return false;
   g->S = S;
   g->d = d;
   g->V = V;
-  g->nchunk = (S + 255) / 256;
-  const int per = (S + g->nchunk - 1) / g->nchunk;
-  g->chunk_n = ((per < 16 ? 16 : per) + 15) / 16 * 16;
-  g->S_pad = g->nchunk * g->chunk_n;
-  if (g->S_pad > 512) return false;
-  g->acc_bufs = 2 * g->S_pad <= 512 ? 2 : 1;
-  uint32_t cols = 32;
-  while (cols < (uint32_t)(g->acc_bufs * g->S_pad)) cols <<= 1;
-  g->tmem_cols = cols;
+  g->pair = S >= LM_PAIR_MIN_S;
+  if (g->pair) {
+    // N of a pair's MMA is a multiple of 32 up to 256
+    g->S_pad = (S + 31) / 32 * 32;
+    if (g->S_pad <= 256) {
+      g->chunk_n = g->S_pad;
+      g->acc_bufs = 2;
+    } else if (g->S_pad <= 384) {
+      g->chunk_n = 512 - g->S_pad;  // double buffered; the rest, at most 256 columns, once
+      g->acc_bufs = 2;
+    } else {
+      g->chunk_n = 256;
+      g->acc_bufs = 1;
+    }
+    g->tmem_cols = 512;
+  } else {
+    g->chunk_n = g->S_pad = ((S < 16 ? 16 : S) + 15) / 16 * 16;
+    g->acc_bufs = 2;
+    uint32_t cols = 32;
+    while (cols < (uint32_t)(2 * g->S_pad)) cols <<= 1;
+    g->tmem_cols = cols;
+  }
   g->ntiles = (V + LM_TILE_V - 1) / LM_TILE_V;
   g->nks = d / LM_TILE_K;
-  const size_t slab = LM_A_BYTES + (size_t)g->S_pad * 128;
-  const size_t fixed = 1024 + 64 * 8 + 16 + (size_t)2 * 4 * g->S_pad * sizeof(float2) +
+  const size_t fixed = 1024 + 80 * 8 + 16 + 4 * LM_TRING + (size_t)2 * 4 * g->S_pad * sizeof(float2) +
                        (size_t)2 * g->S_pad * sizeof(float2) + (size_t)g->S_pad * sizeof(float2) + 32 * 4 + 8 * 64 * 4 + 64 + 128;
-  // several consecutive K-slabs per stage so each row is fetched in longer
-  // runs and the tensor cores get longer bursts per stage; keep at least
-  // three stages in flight
-  g->slabs = 1;
-  for (int sl = 4; sl >= 2; sl >>= 1)
-    if (g->nks % sl == 0 && fixed + 3 * sl * slab <= LM_SMEM_BUDGET) {
-      g->slabs = sl;
-      break;
-    }
-  const size_t stage = (size_t)g->slabs * slab;
-  int st = (int)((LM_SMEM_BUDGET - fixed) / stage);
-  if (st > 8) st = 8;
-  if (st < 2) return false;
-  g->stages = st;
-  g->nst = g->nks / g->slabs;
-  g->smem = fixed + (size_t)st * stage;
+  if (g->pair) {
+    // W comes from HBM and H from L2: H has few stages, W what is left
+    const size_t hslab = (size_t)g->S_pad * 64;
+    g->slabs = 1;
+    g->nst = g->nks;
+    g->hstages = LM_PAIR_HSTAGES;
+    while (g->hstages > 2 && fixed + g->hstages * (hslab + LM_A_BYTES) > LM_SMEM_BUDGET) --g->hstages;
+    int st = (int)((LM_SMEM_BUDGET - fixed - g->hstages * hslab) / LM_A_BYTES);
+    if (st > 12) st = 12;
+    g->stages = st;
+    g->smem = fixed + g->hstages * hslab + (size_t)st * LM_A_BYTES;
+  } else {
+    const size_t slab = LM_A_BYTES + (size_t)g->S_pad * 128;
+    // several consecutive K-slabs per stage so each row is fetched in longer
+    // runs and the tensor cores get longer bursts per stage; keep at least
+    // three stages in flight
+    g->slabs = 1;
+    for (int sl = 4; sl >= 2; sl >>= 1)
+      if (g->nks % sl == 0 && fixed + 3 * sl * slab <= LM_SMEM_BUDGET) {
+        g->slabs = sl;
+        break;
+      }
+    const size_t stage = (size_t)g->slabs * slab;
+    int st = (int)((LM_SMEM_BUDGET - fixed) / stage);
+    if (st > 8) st = 8;
+    if (st < 2) return false;
+    g->stages = st;
+    g->hstages = 0;
+    g->nst = g->nks / g->slabs;
+    g->smem = fixed + (size_t)st * stage;
+  }
   int sms = pced_host::num_sms();
-  g->grid = g->ntiles < sms ? g->ntiles : sms;
-  if (g->grid < 1) g->grid = 1;
+  if (g->pair) {
+    const int pairs = (g->ntiles + 1) / 2;
+    g->grid = 2 * (pairs < sms / 2 ? pairs : sms / 2);
+    if (g->grid < 2) g->grid = 2;
+  } else {
+    g->grid = g->ntiles < sms ? g->ntiles : sms;
+    if (g->grid < 1) g->grid = 1;
+  }
   return true;
 }
 
-// Top-2 over tokens of (value, token) candidates whose token sets are
-// disjoint: (b1, t1) the best (larger value, then lower token), b2 the best
-// value at another token; merges the candidate set (r1, rt, r2) into it.
-__device__ __forceinline__ void top2_merge(float& b1, int& t1, float& b2, float r1, int rt, float r2) {
-  if (r1 > b1 || (r1 == b1 && rt < t1)) {
-    b2 = fmaxf(b1, r2);
-    b1 = r1;
-    t1 = rt;
-  } else {
-    b2 = fmaxf(b2, r1);
+pced_status lm_head_maps(const void* w_unembed, const void* hidden, const LmGeom& g, LmMaps* m) {
+  using pced_host::make_tmap_2d;
+  pced_status st = make_tmap_2d(&m->w, w_unembed, (uint64_t)g.V, (uint64_t)g.d, LM_TILE_V, LM_TILE_K, true);
+  const int share = g.pair ? 2 : 1;  // a CTA of a pair loads half of a chunk's rows
+  for (int c = 0; c < 2 && st == PCED_OK; ++c) {
+    const int n = c == 0 || g.chunk_n == g.S_pad ? g.chunk_n : g.S_pad - g.chunk_n;
+    st = make_tmap_2d(&m->h[c], hidden, (uint64_t)g.S, (uint64_t)g.d, (uint32_t)(n / share), LM_TILE_K, false);
+    if (g.chunk_n == g.S_pad) {
+      m->h[1] = m->h[0];
+      break;
+    }
   }
+  return st;
 }
 
-struct FMax {
-  __device__ __forceinline__ float operator()(float x, float y) const { return fmaxf(x, y); }
-};
-struct FAdd {
-  __device__ __forceinline__ float operator()(float x, float y) const { return x + y; }
-};
-
-// Reduce NB columns held one per register over the 32 lanes (vocabulary rows)
-// of a warp in transposed form: every exchange hands half of the columns still
-// held to the partner lane, so NB columns cost NB - 1 shuffles instead of
-// 5 NB.  The pairing (lane bit 4 first, bit 0 last) is that of a per-column
-// xor tree, so sums round identically.  NB = 32: lane l ends with column l;
-// NB = 16 or 8: full exchanges across the lane bits at and above NB first, so
-// every lane l ends with column l & (NB - 1).
-template <int NB, class Op>
-__device__ __forceinline__ float bfly_reduce(float (&x)[NB], int lane, Op op) {
-#pragma unroll
-  for (int w = 16; w >= NB; w >>= 1) {
-#pragma unroll
-    for (int i = 0; i < NB; ++i) x[i] = op(x[i], __shfl_xor_sync(0xffffffffu, x[i], w));
-  }
-#pragma unroll
-  for (int w = NB / 2; w >= 1; w >>= 1) {
-    const bool hi = (lane & w) != 0;
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const float send = hi ? x[i] : x[i + w];
-      const float keep = hi ? x[i + w] : x[i];
-      x[i] = op(keep, __shfl_xor_sync(0xffffffffu, send, w));
-    }
-  }
-  return x[0];
-}
-
-// Top-2 over the 32 lanes (vocabulary rows) of NB columns held one per
-// register, in the transposed form of bfly_reduce: (best value, its token,
-// best value at another token) travel together, ties to the lower token.
-// Lane l ends with column l & (NB - 1).  `tok` is this lane's token.
-template <int NB>
-__device__ __forceinline__ void bfly_top2(const float (&u)[NB], int tok, int lane, float& r1, int& rt, float& r2) {
-  constexpr int K = NB == 32 ? 16 : NB;  // slots after the first level
-  float b1[K], b2[K];
-  int bt[K];
-  const int ptok = tok + ((lane ^ 16) - lane);  // the row across lane bit 4
-  const bool hi16 = (lane & 16) != 0;
-#pragma unroll
-  for (int i = 0; i < K; ++i) {
-    // NB = 32: the first halving level; NB <= 16: a full exchange
-    const float send = NB == 32 ? (hi16 ? u[i] : u[(i + 16) % NB]) : u[i];
-    const float keep = NB == 32 ? (hi16 ? u[(i + 16) % NB] : u[i]) : u[i];
-    const float o = __shfl_xor_sync(0xffffffffu, send, 16);
-    const bool take = o > keep || (o == keep && ptok < tok);
-    b1[i] = take ? o : keep;
-    bt[i] = take ? ptok : tok;
-    b2[i] = take ? keep : o;
-  }
-  // NB = 8: one more full exchange, across lane bit 3
-#pragma unroll
-  for (int w = 8; w >= NB; w >>= 1) {
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-      const float o1 = __shfl_xor_sync(0xffffffffu, b1[i], w), o2 = __shfl_xor_sync(0xffffffffu, b2[i], w);
-      const int ot = __shfl_xor_sync(0xffffffffu, bt[i], w);
-      top2_merge(b1[i], bt[i], b2[i], o1, ot, o2);
-    }
-  }
-#pragma unroll
-  for (int w = (NB == 32 ? 8 : NB / 2); w >= 1; w >>= 1) {
-    const bool hi = (lane & w) != 0;
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const float s1 = hi ? b1[i] : b1[i + w], s2 = hi ? b2[i] : b2[i + w];
-      const int st = hi ? bt[i] : bt[i + w];
-      float k1 = hi ? b1[i + w] : b1[i], k2 = hi ? b2[i + w] : b2[i];
-      int kt = hi ? bt[i + w] : bt[i];
-      const float o1 = __shfl_xor_sync(0xffffffffu, s1, w), o2 = __shfl_xor_sync(0xffffffffu, s2, w);
-      const int ot = __shfl_xor_sync(0xffffffffu, st, w);
-      top2_merge(k1, kt, k2, o1, ot, o2);
-      b1[i] = k1;
-      bt[i] = kt;
-      b2[i] = k2;
-    }
-  }
-  r1 = b1[0];
-  rt = bt[0];
-  r2 = b2[0];
-}
-
-// Epilogue of NB accumulator columns c0.. (c0 a multiple of NB) of one
-// warp's 32 vocabulary rows: mode 0 stores the logits; both modes record the
-// per-column (max, sum of exp) of the 32 rows; mode 1 also records per expert
-// column the max of u_k = (1 + beta) z_k - beta z_0, its first (lowest)
-// vocabulary index and the best value at another index.  `bc` is this warp's
-// broadcast buffer; z_am carries the row's amateur logit from its query's
-// first column to the expert columns; ccoef / cmask hold each column's
-// (1 + beta, beta) and the amateur / expert column bits of each 32-column
-// block (the same for every tile).
-template <int NB>
-__device__ __forceinline__ void epi_block(const LmArgs& a, uint32_t taddr, int c0, int v, bool valid, int lane,
-                                          int q, float* bc, float2* wst, float2* wag, float* wu2, const float2* ccoef,
-                                          const uint32_t* cmask, float& z_am) {
-  const int S = a.S, S_pad = a.S_pad;
-  float z[NB], t[NB];
-  if (NB == 32)
-    tmem_ld32(taddr, z);
-  else if (NB == 16)
-    tmem_ld16(taddr, z);
-  else
-    tmem_ld8(taddr, z);
-  if (a.mode == 0 && valid) {
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-      if (c0 + i < S) a.logits[(int64_t)(c0 + i) * a.V + v] = z[i];
-  }
-#pragma unroll
-  for (int i = 0; i < NB; ++i) t[i] = valid ? z[i] : -INFINITY;
-  float u[NB];
-  const uint32_t em = a.mode == 1 ? cmask[16 + (c0 >> 5)] >> (c0 & 31) : 0u;
-  if (a.mode == 1) {
-    const uint32_t am = cmask[c0 >> 5] >> (c0 & 31);
-    float za = z_am;
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-      if ((am >> i) & 1u) za = z[i];
-      const float2 cf = ccoef[c0 + i];
-      u[i] = valid && ((em >> i) & 1u) ? cf.x * z[i] - cf.y * za : -INFINITY;
-    }
-    z_am = za;
-  }
-  const float m = bfly_reduce<NB>(t, lane, FMax());
-  float b1 = -INFINITY, b2 = -INFINITY;
-  int bt = 0;
-  if (a.mode == 1) bfly_top2<NB>(u, v, lane, b1, bt, b2);
-  const int li = lane & (NB - 1), mycol = c0 + li;
-  if (lane < NB) bc[lane] = m;
-  __syncwarp();
-#pragma unroll
-  for (int i = 0; i < NB; ++i) t[i] = valid ? __expf(z[i] - bc[i]) : 0.f;
-  const float sm = bfly_reduce<NB>(t, lane, FAdd());
-  if (lane < NB && mycol < S) {
-    wst[q * S_pad + mycol] = make_float2(m, sm);
-    if ((em >> li) & 1u) {
-      wag[q * S_pad + mycol] = make_float2(b1, __int_as_float(bt));
-      wu2[q * S_pad + mycol] = b2;
-    }
-  }
-  __syncwarp();
+LmArgs lm_args(const LmGeom& g) {
+  LmArgs a = {};
+  a.S = g.S;
+  a.V = g.V;
+  a.ntiles = g.ntiles;
+  a.nks = g.nks;
+  a.slabs = g.slabs;
+  a.nst = g.nst;
+  a.stages = g.stages;
+  a.hstages = g.hstages;
+  a.acc_bufs = g.acc_bufs;
+  a.S_pad = g.S_pad;
+  a.chunk_n = g.chunk_n;
+  a.tmem_cols = g.tmem_cols;
+  return a;
 }
 
 // The MMAs of one stage of SL K-slabs (single N chunk), fully unrolled: the
 // start-address field of a K-major SW128 descriptor advances by 2 per 16-wide
 // K-step and by the slab size >> 4 per slab.
 template <int SL>
-__device__ __forceinline__ void umma_slabs(uint32_t dcol, uint64_t ad0, uint64_t bd0, uint32_t bstep, uint32_t idesc,
+__device__ __forceinline__ void umma_slabs(uint32_t on, uint32_t dcol, uint64_t ad0, uint64_t bd0, uint32_t bstep, uint32_t idesc,
                                            bool first) {
 #pragma unroll
   for (int j = 0; j < SL; ++j)
 #pragma unroll
     for (int k = 0; k < LM_TILE_K / 16; ++k)
-      umma_bf16(dcol, ad0 + (uint64_t)(j * (LM_A_BYTES >> 4) + 2 * k), bd0 + (uint64_t)(j * bstep + 2 * k), idesc,
+      umma_bf16(on, dcol, ad0 + (uint64_t)(j * (LM_A_BYTES >> 4) + 2 * k), bd0 + (uint64_t)(j * bstep + 2 * k), idesc,
                 !(first && j == 0 && k == 0));
 }
 
@@ -268,14 +172,14 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + (bar_drain + 8 - base));
   int32_t* tring = reinterpret_cast<int32_t*>(tmem_slot + 4);  // [LM_TRING] claimed tiles, producer -> MMA warp
   int32_t* acc_tile = tring + LM_TRING;                        // [2] tile of each accumulator, MMA warp -> epilogue
-  float2* wst = reinterpret_cast<float2*>(gbase + (bar_drain + 8 - base) + 96);  // [4][S_pad] per-warp stats
+  float2* wst = reinterpret_cast<float2*>(gbase + (bar_drain + 8 - base) + 32 + 4 * LM_TRING);  // [4][S_pad] per-warp stats
   float2* wag = wst + 4 * S_pad;                                                  // [4][S_pad] per-warp argmax
   float* wu2 = reinterpret_cast<float*>(wag + 4 * S_pad);                         // [4][S_pad] per-warp runner-up
   float2* ccoef = wag + 6 * S_pad;                                 // [S_pad] (1 + beta, beta) per column
   uint32_t* cmask = reinterpret_cast<uint32_t*>(ccoef + S_pad);     // [2][16] amateur / expert column bits
   float* bc = reinterpret_cast<float*>(cmask + 32);                // [8][64] per-warp column broadcast
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) {
       mbar_init(bar_full + 8 * i, 1);
@@ -294,181 +198,139 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
     tma_prefetch_desc(&wmap);
     tma_prefetch_desc(&hmap);
   }
-  if (a.pdl) pdl_launch_dependents();
+  pdl_launch_dependents();
   if (warp == 1) {
     tmem_alloc(smem_u32(tmem_slot), a.tmem_cols);
     tmem_relinquish();
   }
-  if (a.mode == 1) {
-    // per column: expert columns carry (1 + beta_k, beta_k), the amateur
-    // column of each query starts its group; bit i of block kb is column 32 kb + i
-    const int n1 = a.N + 1;
-    for (int c = tid; c < S_pad; c += LM_THREADS) {
-      const int j = c % n1, bq = c / n1;
-      const float bt = c < a.S && j > 0 ? a.beta[bq * a.N + j - 1] : 0.f;
-      ccoef[c] = make_float2(1.f + bt, bt);
-    }
-    if (warp == 0)
-      for (int kb = 0; kb < 16; ++kb) {
-        const int c = 32 * kb + lane;
-        const bool in = c < a.S;
-        const uint32_t am = __ballot_sync(0xffffffffu, in && c % n1 == 0);
-        const uint32_t em = __ballot_sync(0xffffffffu, in && c % n1 != 0);
-        if (lane == 0) {
-          cmask[kb] = am;
-          cmask[16 + kb] = em;
-        }
-      }
-  }
+  if (a.mode == 1) column_tables(a, tid, ccoef, cmask);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const int ntiles = a.ntiles, nst = a.nst;
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA
-    if (lane == 0) {
-      const uint64_t pol_w = policy_evict_first(), pol_h = policy_evict_last();
-      // Tiles are claimed from a global counter, so CTAs that start early (as
-      // the previous kernel's CTAs leave their SMs) take more of them.  The
-      // claimed ids reach the MMA warp through tring (written before the
-      // arrive on the full barrier of the tile's first stage); -1 ends.
-      int tile = -1, ks = 0;
-      uint32_t tseq = 0;
-      auto claim = [&]() {
-        const int t = atomicAdd(a.tile_ctr, 1);
-        tile = t < ntiles ? t : -1;
-        tring[tseq % LM_TRING] = tile;
-        ++tseq;
-        ks = 0;
-      };
-      auto load_w = [&](uint32_t st) {
-        const uint32_t fb = bar_full + 8 * st, sa = base + st * st_bytes;
-        mbar_arrive_expect_tx(fb, st_bytes);
-        // consecutive K-slabs of the same 128 rows back to back: longer runs per row
-        for (int j = 0; j < SL; ++j)
-          tma_load_2d(sa + j * LM_A_BYTES, &wmap, fb, (ks * SL + j) * LM_TILE_K, tile * LM_TILE_V, pol_w);
-      };
-      auto load_h = [&](uint32_t st, int kss) {
-        const uint32_t fb = bar_full + 8 * st, sb = base + st * st_bytes + SL * LM_A_BYTES;
-        for (int j = 0; j < SL; ++j)
-          for (int c = 0; c < a.nchunk; ++c)
-            tma_load_2d(sb + j * b_bytes + c * a.chunk_n * 128, &hmap, fb, (kss * SL + j) * LM_TILE_K,
-                        c * a.chunk_n, pol_h);
-      };
-      claim();
-      uint32_t it = 0;
-      // With programmatic dependent launch the weights of the first stages
-      // stream while the previous kernel (which writes H) finishes.
-      if (a.pdl) {
-        int pre_ks[8];
-        while (tile >= 0 && it < (uint32_t)stages) {
-          load_w(it);
-          pre_ks[it++] = ks;
-          if (++ks == nst) claim();
-        }
-        pdl_wait();
-        for (uint32_t i = 0; i < it; ++i) load_h(i, pre_ks[i]);
+    const uint32_t on = elect_one();
+    const uint64_t pol_w = policy_evict_first(), pol_h = policy_evict_last();
+    // Tiles are claimed from a global counter, so CTAs that start early (as
+    // the previous kernel's CTAs leave their SMs) take more of them.  The
+    // claimed ids reach the MMA warp through tring (written before the
+    // arrive on the full barrier of the tile's first stage); -1 ends.
+    int tile = -1, ks = 0;
+    uint32_t tseq = 0;
+    auto claim = [&]() {
+      int t = -1;
+      if (lane == 0) {
+        t = atomicAdd(a.tile_ctr, 1);
+        if (t >= ntiles) t = -1;
+        tring[tseq % LM_TRING] = t;
       }
-      bool ok = true;
-      while (tile >= 0) {
-        const uint32_t st = it % stages, ph = (it / stages) & 1u;
-        if (!mbar_wait(bar_empty + 8 * st, ph ^ 1u, a.status)) {
-          ok = false;
-          break;
-        }
-        load_w(st);
-        load_h(st, ks);
-        ++it;
+      tile = __shfl_sync(0xffffffffu, t, 0);
+      ++tseq;
+      ks = 0;
+    };
+    auto load_w = [&](uint32_t st) {
+      const uint32_t fb = bar_full + 8 * st, sa = base + st * st_bytes;
+      mbar_arrive_expect_tx_if(on, fb, st_bytes);
+      // consecutive K-slabs of the same 128 rows back to back: longer runs per row
+      for (int j = 0; j < SL; ++j)
+        tma_load_2d(on, sa + j * LM_A_BYTES, &wmap, fb, (ks * SL + j) * LM_TILE_K, tile * LM_TILE_V, pol_w);
+    };
+    auto load_h = [&](uint32_t st, int kss) {
+      const uint32_t fb = bar_full + 8 * st, sb = base + st * st_bytes + SL * LM_A_BYTES;
+      for (int j = 0; j < SL; ++j)
+        tma_load_2d(on, sb + j * b_bytes, &hmap, fb, (kss * SL + j) * LM_TILE_K, 0, pol_h);
+    };
+    claim();
+    uint32_t it = 0;
+    // With programmatic dependent launch the weights of the first stages
+    // stream while the previous kernel (which writes H) finishes; a tile has
+    // nst stages, so stage i of these belongs to stage i % nst of its tile.
+    if (a.pdl) {
+      while (tile >= 0 && it < (uint32_t)stages) {
+        load_w(it++);
         if (++ks == nst) claim();
       }
-      if (ok) {
-        // end marker: a phase of the next stage's full barrier without data
-        const uint32_t st = it % stages, ph = (it / stages) & 1u;
-        if (mbar_wait(bar_empty + 8 * st, ph ^ 1u, a.status)) mbar_arrive(bar_full + 8 * st);
-      } else {
-        for (uint32_t j = (it >= (uint32_t)stages ? it - stages : 0); j < it; ++j)
-          mbar_wait(bar_full + 8 * (j % stages), (j / stages) & 1u, a.status);
+      pdl_wait();
+      for (uint32_t i = 0; i < it; ++i) load_h(i, (int)(i % (uint32_t)nst));
+    }
+    bool ok = true;
+    uint32_t st = it == (uint32_t)stages ? 0 : it, ph = it == (uint32_t)stages ? 1 : 0;
+    while (tile >= 0) {
+      if (!mbar_wait_warp(bar_empty + 8 * st, ph ^ 1u, a.status)) {
+        ok = false;
+        break;
       }
+      load_w(st);
+      load_h(st, ks);
+      ++it;
+      if (++st == (uint32_t)stages) {
+        st = 0;
+        ph ^= 1u;
+      }
+      if (++ks == nst) claim();
+    }
+    if (ok) {
+      // end marker: a phase of the next stage's full barrier without data
+      if (mbar_wait_warp(bar_empty + 8 * st, ph ^ 1u, a.status) && lane == 0) mbar_arrive(bar_full + 8 * st);
+    } else {
+      for (uint32_t j = (it >= (uint32_t)stages ? it - stages : 0); j < it; ++j)
+        mbar_wait_warp(bar_full + 8 * (j % stages), (j / stages) & 1u, a.status);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(LM_TILE_V, a.chunk_n);
-      uint32_t it = 0, acc = 0, tseq = 0;
-      bool ok = true;
-      for (;; ++acc) {
-        const uint32_t buf = acc % a.acc_bufs, aph = (acc / a.acc_bufs) & 1u;
-        // the next tile's first stage (or the end marker) tells which tile it is
-        {
-          const uint32_t st = it % stages, ph = (it / stages) & 1u;
-          if (!mbar_wait(bar_full + 8 * st, ph, a.status)) {
-            ok = false;
-            break;
-          }
-        }
-        const int tile = tring[tseq % LM_TRING];
-        ++tseq;
-        if (!mbar_wait(bar_tempty + 8 * buf, aph ^ 1u, a.status)) {
+    const uint32_t on = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(LM_TILE_V, a.chunk_n);
+    uint32_t acc = 0, tseq = 0, st = 0, ph = 0;
+    bool ok = true;
+    for (;; ++acc) {
+      const uint32_t buf = acc & 1u, aph = (acc >> 1) & 1u;
+      // the next tile's first stage (or the end marker) tells which tile it is
+      if (!mbar_wait_warp(bar_full + 8 * st, ph, a.status)) break;
+      const int tile = __shfl_sync(0xffffffffu, tring[tseq % LM_TRING], 0);
+      ++tseq;
+      if (!mbar_wait_warp(bar_tempty + 8 * buf, aph ^ 1u, a.status)) break;
+      if (lane == 0) {
+        acc_tile[buf] = tile;
+        mbar_arrive(bar_tid + 8 * buf);
+      }
+      __syncwarp();
+      if (tile < 0) break;
+      tc_fence_after();
+      const uint32_t dcol = tmem_base + buf * S_pad;
+      for (int ks = 0; ks < nst; ++ks) {
+        if (ks > 0 && !mbar_wait_warp(bar_full + 8 * st, ph, a.status)) {
           ok = false;
           break;
         }
-        acc_tile[buf] = tile;
-        mbar_arrive(bar_tid + 8 * buf);
-        if (tile < 0) break;
         tc_fence_after();
-        const uint32_t dcol = tmem_base + buf * S_pad;
-        for (int ks = 0; ks < nst; ++ks, ++it) {
-          const uint32_t st = it % stages, ph = (it / stages) & 1u;
-          if (ks > 0 && !mbar_wait(bar_full + 8 * st, ph, a.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sa = base + st * st_bytes, sb = sa + SL * LM_A_BYTES;
-          // descriptors are built once per stage; a K-step moves the start
-          // address field (bytes >> 4) by 2, a slab by its size >> 4
-          const uint64_t ad0 = umma_desc_sw128(sa), bd0 = umma_desc_sw128(sb);
-          if (a.nchunk == 1 && (SL == 4 || SL == 2 || SL == 1)) {
-            const uint32_t bstep = b_bytes >> 4;
-            const bool first = ks == 0;
-            if (SL == 4)
-              umma_slabs<4>(dcol, ad0, bd0, bstep, idesc, first);
-            else if (SL == 2)
-              umma_slabs<2>(dcol, ad0, bd0, bstep, idesc, first);
-            else
-              umma_slabs<1>(dcol, ad0, bd0, bstep, idesc, first);
-          } else if (a.nchunk == 2 && SL == 1) {
-            // more than 256 hidden rows: two N chunks per K-step, unrolled
-            // (the issuing thread, not the data, set the pace with a loop here)
-            const uint32_t coff = (uint32_t)(a.chunk_n * 128) >> 4, dc1 = dcol + a.chunk_n;
-#pragma unroll
-            for (int k = 0; k < LM_TILE_K / 16; ++k) {
-              umma_bf16(dcol, ad0 + 2 * k, bd0 + 2 * k, idesc, (ks | k) != 0);
-              umma_bf16(dc1, ad0 + 2 * k, bd0 + coff + 2 * k, idesc, (ks | k) != 0);
-            }
-          } else {
-            for (int j = 0; j < SL; ++j) {
-#pragma unroll
-              for (int k = 0; k < LM_TILE_K / 16; ++k) {
-                const uint64_t ad = ad0 + (uint64_t)(j * (LM_A_BYTES >> 4) + 2 * k);
-                for (int c = 0; c < a.nchunk; ++c)
-                  umma_bf16(dcol + c * a.chunk_n, ad, bd0 + (uint64_t)((j * b_bytes + c * a.chunk_n * 128) >> 4) + 2 * k,
-                            idesc, (ks | j | k) != 0);
-              }
-            }
-          }
-          umma_commit(bar_empty + 8 * st);
+        const uint32_t sa = base + st * st_bytes, sb = sa + SL * LM_A_BYTES;
+        // descriptors are built once per stage; a K-step moves the start
+        // address field (bytes >> 4) by 2, a slab by its size >> 4
+        const uint64_t ad0 = umma_desc_sw128(sa), bd0 = umma_desc_sw128(sb);
+        const uint32_t bstep = b_bytes >> 4;
+        const bool first = ks == 0;
+        if (SL == 4)
+          umma_slabs<4>(on, dcol, ad0, bd0, bstep, idesc, first);
+        else if (SL == 2)
+          umma_slabs<2>(on, dcol, ad0, bd0, bstep, idesc, first);
+        else
+          umma_slabs<1>(on, dcol, ad0, bd0, bstep, idesc, first);
+        umma_commit(on, bar_empty + 8 * st);
+        if (++st == (uint32_t)stages) {
+          st = 0;
+          ph ^= 1u;
         }
-        if (!ok) break;
-        umma_commit(bar_tfull + 8 * buf);
       }
-      // all issued MMAs complete before TMEM is released
-      umma_commit(bar_drain);
-      mbar_wait(bar_drain, 0, a.status);
+      if (!ok) break;
+      umma_commit(on, bar_tfull + 8 * buf);
     }
+    // all issued MMAs complete before TMEM is released
+    umma_commit(on, bar_drain);
+    mbar_wait_warp(bar_drain, 0, a.status);
     __syncwarp();
   } else {
     // ----------------------------------------------------------- epilogue
@@ -477,7 +339,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
     const int S = a.S, n1 = a.N + 1;
     uint32_t ephase = 0;
     for (uint32_t acc = 0;; ++acc) {
-      const uint32_t buf = acc % a.acc_bufs, aph = (acc / a.acc_bufs) & 1u;
+      const uint32_t buf = acc & 1u, aph = (acc >> 1) & 1u;
       if (!mbar_wait(bar_tid + 8 * buf, aph, a.status)) break;
       const int tile = acc_tile[buf];
       if (tile < 0) break;
@@ -507,30 +369,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
       tc_fence_before();
       mbar_arrive(bar_tempty + 8 * buf);
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
-      // this tile's records: the four lane quarters' results folded in a fixed
-      // order, stored per tile so the cross-tile merge order does not depend
-      // on which CTA took the tile
       const bool tile_ok = PCED_IN_BOUNDS(tile < ntiles, a.status);
-      for (int col = etid; col < S && tile_ok; col += LM_EPI_THREADS) {
-        float cm = -INFINITY, cs = 0.f;
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) {
-          const float2 r = wst[qq * S_pad + col];
-          lse_merge(cm, cs, r.x, r.y);
-        }
-        a.rec_stats[(int64_t)col * ntiles + tile] = make_float2(cm, cs);
-        if (a.mode == 1 && col % n1 != 0) {
-          float bu = -INFINITY, b2 = -INFINITY;
-          int bv = 0x7fffffff;
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) {
-            const float2 r = wag[qq * S_pad + col];
-            top2_merge(bu, bv, b2, r.x, __float_as_int(r.y), wu2[qq * S_pad + col]);
-          }
-          a.rec_arg[(int64_t)col * ntiles + tile] = make_float2(bu, __int_as_float(bv));
-          a.rec_u2[(int64_t)col * ntiles + tile] = b2;
-        }
-      }
+      if (tile_ok) fold_tile(a, tile, etid, wst, wag, wu2);
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
     }
   }
@@ -542,8 +382,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
   }
 }
 
-cudaError_t lm_head_launch(const CUtensorMap& wmap, const CUtensorMap& hmap, const LmGeom& g, const LmArgs& a,
-                           cudaStream_t stream) {
+cudaError_t lm_head_launch(const LmMaps& m, const LmGeom& g, const LmArgs& a, cudaStream_t stream) {
+  if (g.pair) return lm_head_pair_launch(m, g, a, stream);
   // the shared-memory limit is an attribute of the kernel on each device
   static bool configured[64];
   int dev = 0;
@@ -555,17 +395,8 @@ cudaError_t lm_head_launch(const CUtensorMap& wmap, const CUtensorMap& hmap, con
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g.grid);
-  cfg.blockDim = dim3(LM_THREADS);
-  cfg.dynamicSmemBytes = g.smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = a.pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, lm_head_kernel, wmap, hmap, a);
+  return pced_host::launch_kernel(lm_head_kernel, dim3(g.grid), LM_THREADS, g.smem, stream, a.pdl != 0,
+                                  m.w, m.h[0], a);
 }
 
 // ------------------------------------------------------------ mode-0 finish
@@ -889,37 +720,19 @@ extern "C" pced_status pced_lm_head_logprobs(const void* hidden, const void* w_u
   if (((uintptr_t)workspace) & 255u || workspace_bytes < pced_lm_head_workspace_size(S, V))
     return fail(PCED_ERR_WORKSPACE, "pced_lm_head_logprobs: workspace too small or misaligned");
   if (num_sms() <= 0) return fail(PCED_ERR_NO_DEVICE, "pced_lm_head_logprobs: no CUDA device");
-  CUtensorMap wmap, hmap;
-  pced_status st = make_tmap_2d(&wmap, w_unembed, (uint64_t)V, (uint64_t)d, LM_TILE_V, LM_TILE_K, true);
-  if (st != PCED_OK) return st;
-  st = make_tmap_2d(&hmap, hidden, (uint64_t)S, (uint64_t)d, (uint32_t)g.chunk_n, LM_TILE_K, false);
+  LmMaps maps;
+  const pced_status st = lm_head_maps(w_unembed, hidden, g, &maps);
   if (st != PCED_OK) return st;
   Carver cv((char*)workspace + 256);
-  LmArgs a = {};
-  a.mode = 0;
-  a.S = S;
-  a.N = 0;
-  a.V = V;
-  a.ntiles = g.ntiles;
-  a.nks = g.nks;
-  a.slabs = g.slabs;
-  a.nst = g.nst;
-  a.stages = g.stages;
-  a.acc_bufs = g.acc_bufs;
-  a.S_pad = g.S_pad;
-  a.nchunk = g.nchunk;
-  a.chunk_n = g.chunk_n;
-  a.tmem_cols = g.tmem_cols;
+  LmArgs a = lm_args(g);
   a.logits = logprobs;
   a.rec_stats = cv.take<float2>((size_t)S * g.ntiles);
-  a.rec_arg = nullptr;
-  a.beta = nullptr;
   a.status = (int*)workspace;
   a.tile_ctr = (int*)workspace + 1;  // tile counter, zeroed here
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaMemsetAsync(a.tile_ctr, 0, sizeof(int), s);
   if (e != cudaSuccess) return cuda_status(e, "lm head tile counter");
-  e = lm_head_launch(wmap, hmap, g, a, s);
+  e = lm_head_launch(maps, g, a, s);
   if (e != cudaSuccess) return cuda_status(e, "lm head launch");
   e = lm_lse_finalize_launch(logprobs, a.rec_stats, lse, S, V, g.ntiles, s);
   if (e != cudaSuccess) return cuda_status(e, "lse finalize launch");

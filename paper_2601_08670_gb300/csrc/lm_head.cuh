@@ -11,10 +11,18 @@ constexpr int LM_TILE_V = 128;   // vocabulary rows per tile (UMMA M)
 constexpr int LM_TILE_K = 64;    // hidden elements per stage (one 128-byte swizzle row)
 constexpr int LM_MAX_S = 512;
 constexpr int LM_MAX_N1 = 256;   // experts + amateur per query in the selection kernels
-constexpr int LM_TRING = 16;     // claimed-tile ring between the TMA and MMA warps (> stages + 2 tiles in flight)
+constexpr int LM_TRING = 32;     // claimed-tile ring between the TMA and the other warps (> stages + 3 tiles in flight)
+
+constexpr int LM_A_BYTES = LM_TILE_V * LM_TILE_K * 2;  // 16 KB
+constexpr size_t LM_SMEM_BUDGET = 227 * 1024;
+// From this many hidden rows on a tile is taken by a pair of CTAs
+// (lm_head_pair.cu), below by one (lm_head.cu): equal at 128 rows, 207 against
+// 205 us at 160, 219 against 216 us at 192 (d = 4096, V = 128256).
+constexpr int LM_PAIR_MIN_S = 161;
 
 struct LmGeom {
-  int32_t S, S_pad, nchunk, chunk_n, d, V, ntiles, nks, slabs, nst, stages, acc_bufs, grid;
+  bool pair;
+  int32_t S, S_pad, chunk_n, d, V, ntiles, nks, slabs, nst, stages, hstages, acc_bufs, grid;
   uint32_t tmem_cols;
   size_t smem;
 };
@@ -23,7 +31,9 @@ bool lm_geometry(int32_t S, int32_t d, int32_t V, LmGeom* g);
 
 struct LmArgs {
   int mode;  // 0: write logits[S][V]; 1: contrastive records (needs N, beta)
-  int32_t S, N, V, ntiles, nks, slabs, nst, stages, acc_bufs, S_pad, nchunk, chunk_n;
+  int32_t S, N, V, ntiles, nks, slabs, nst, stages, acc_bufs, S_pad;
+  int32_t hstages;    // pair: stages of the H ring (stages: of the W ring)
+  int32_t chunk_n;    // accumulator columns of the first N chunk (pair: S_pad - chunk_n in a second one)
   uint32_t tmem_cols;
   float* logits;      // mode 0
   float2* rec_stats;  // [S][ntiles] (max z, sum exp(z - max)) of each vocabulary tile
@@ -35,8 +45,13 @@ struct LmArgs {
   int* status;
 };
 
-cudaError_t lm_head_launch(const CUtensorMap& wmap, const CUtensorMap& hmap, const LmGeom& g, const LmArgs& a,
-                           cudaStream_t stream);
+struct LmMaps {
+  CUtensorMap w, h[2];  // W tiles; H rows of the N chunks
+};
+pced_status lm_head_maps(const void* w_unembed, const void* hidden, const LmGeom& g, LmMaps* m);
+LmArgs lm_args(const LmGeom& g);  // the geometry's fields; the others zero
+cudaError_t lm_head_launch(const LmMaps& m, const LmGeom& g, const LmArgs& a, cudaStream_t stream);
+cudaError_t lm_head_pair_launch(const LmMaps& m, const LmGeom& g, const LmArgs& a, cudaStream_t stream);
 // mode-0 finish: lse[s] from the tile records, logits -> log-probs in place
 cudaError_t lm_lse_finalize_launch(float* logits, const float2* rec_stats, float* lse, int32_t S, int32_t V,
                                    int32_t nrec, cudaStream_t stream);

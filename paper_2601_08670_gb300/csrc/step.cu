@@ -222,12 +222,12 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   const int32_t S = dm.B * (dm.N + 1), d = dm.Hq * dm.D, G = dm.Hq / dm.Hkv;
 
   const StepLayout W = step_layout(&dm, p->workspace);
-  CUtensorMap kmap, vmap, wmap, hmap;
+  CUtensorMap kmap, vmap;
+  LmMaps maps;
   const uint64_t rows = (uint64_t)dm.L * (uint64_t)(p->layer_elems / dm.D);
   pced_status st = make_tmap_kv(&kmap, p->k_cache, rows, (uint32_t)dm.D, ATT_BLOCK_N);
   if (st == PCED_OK) st = make_tmap_kv(&vmap, p->v_cache, rows, (uint32_t)dm.D, ATT_BLOCK_N);
-  if (st == PCED_OK) st = make_tmap_2d(&wmap, p->w_unembed, (uint64_t)dm.V, (uint64_t)d, LM_TILE_V, LM_TILE_K, true);
-  if (st == PCED_OK) st = make_tmap_2d(&hmap, W.h, (uint64_t)S, (uint64_t)d, (uint32_t)g.chunk_n, LM_TILE_K, false);
+  if (st == PCED_OK) st = lm_head_maps(p->w_unembed, W.h, g, &maps);
   if (st != PCED_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   const bool dyn = p->beta_from_step != 0;
@@ -310,28 +310,14 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   // fused LM head with that beta or the aggregation kernels
   const float* beta = p->beta;
   if (dyn || agg) {
-    LmArgs lz = {};
-    lz.mode = 0;
-    lz.S = S;
-    lz.N = 0;
-    lz.V = dm.V;
-    lz.ntiles = g.ntiles;
-    lz.nks = g.nks;
-    lz.slabs = g.slabs;
-    lz.nst = g.nst;
-    lz.stages = g.stages;
-    lz.acc_bufs = g.acc_bufs;
-    lz.S_pad = g.S_pad;
-    lz.nchunk = g.nchunk;
-    lz.chunk_n = g.chunk_n;
-    lz.tmem_cols = g.tmem_cols;
+    LmArgs lz = lm_args(g);
     lz.logits = W.lp;
     lz.rec_stats = W.lm_stats;
     lz.tile_ctr = W.lm_tile_ctr;
     lz.status = W.status;
     lz.pdl = timed ? 0 : 1;  // streams weights while the attention kernel finishes
     ranges.next("lm_head");
-    e = lm_head_launch(wmap, hmap, g, lz, s);
+    e = lm_head_launch(maps, g, lz, s);
     if (e == cudaSuccess) e = mark();
     // MoE / PoE alone need no log-probabilities (the aggregation kernels
     // read the raw logits and form the rows' log-sum-exps themselves); beta
@@ -403,21 +389,9 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     return PCED_OK;
   }
 
-  LmArgs la = {};
+  LmArgs la = lm_args(g);
   la.mode = 1;
-  la.S = S;
   la.N = dm.N;
-  la.V = dm.V;
-  la.ntiles = g.ntiles;
-  la.nks = g.nks;
-  la.slabs = g.slabs;
-  la.nst = g.nst;
-  la.stages = g.stages;
-  la.acc_bufs = g.acc_bufs;
-  la.S_pad = g.S_pad;
-  la.nchunk = g.nchunk;
-  la.chunk_n = g.chunk_n;
-  la.tmem_cols = g.tmem_cols;
   la.rec_stats = W.lm_stats;
   la.rec_arg = W.lm_arg;
   la.rec_u2 = W.lm_u2;
@@ -426,7 +400,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   la.status = W.status;
   la.pdl = (timed || dyn) ? 0 : 1;  // stage events between the launches would break the overlap
   ranges.next("lm_head");
-  e = lm_head_launch(wmap, hmap, g, la, s);
+  e = lm_head_launch(maps, g, la, s);
   if (e == cudaSuccess) e = mark();
   if (e != cudaSuccess) return cuda_status(e, "lm head launch");
 
