@@ -400,19 +400,14 @@ cudaError_t lm_head_launch(const LmMaps& m, const LmGeom& g, const LmArgs& a, cu
 }
 
 // ------------------------------------------------------------ mode-0 finish
-// grid (chunks, S): every CTA of row s forms lse[s] from the row's tile
-// records (the same fixed order in each) and turns its chunk of logits into
-// log-probabilities in place; chunk 0 stores lse.
-constexpr int LSE_CHUNK = 8192;  // (144 CTAs for 9 rows of 128K entries)
+constexpr int LSE_THREADS = 256;
 
-__global__ void __launch_bounds__(256) lm_lse_finalize_kernel(float* logits, const float2* rec_stats, float* lse,
-                                                              int32_t V, int32_t nrec) {
-  const int c = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
-  __shared__ float2 red[8];
-  __shared__ float Ls;
+// log-sum-exp of row s from its tile records (fixed order), in every thread
+__device__ __forceinline__ float row_lse(const float2* rec, int32_t nrec, float2* red, float* Ls) {
+  const int tid = threadIdx.x;
   float M = -INFINITY, sum = 0.f;
-  for (int t = tid; t < nrec; t += 256) {
-    const float2 r = rec_stats[(int64_t)s * nrec + t];
+  for (int t = tid; t < nrec; t += LSE_THREADS) {
+    const float2 r = rec[t];
     lse_merge(M, sum, r.x, r.y);
   }
 #pragma unroll
@@ -424,22 +419,69 @@ __global__ void __launch_bounds__(256) lm_lse_finalize_kernel(float* logits, con
   __syncthreads();
   if (tid == 0) {
     float m = -INFINITY, su = 0.f;
-    for (int w = 0; w < 8; ++w) lse_merge(m, su, red[w].x, red[w].y);
-    Ls = m + logf(su);
-    if (c == 0) lse[s] = Ls;
+    for (int w = 0; w < LSE_THREADS / 32; ++w) lse_merge(m, su, red[w].x, red[w].y);
+    *Ls = m + logf(su);
   }
   __syncthreads();
-  const float L = Ls;
-  float* row = logits + (int64_t)s * V;
-  const int v1 = min(V, (c + 1) * LSE_CHUNK);
-  for (int v = c * LSE_CHUNK + tid; v < v1; v += 256) row[v] -= L;
+  return *Ls;
 }
 
+__global__ void __launch_bounds__(LSE_THREADS) lm_lse_kernel(const float2* rec_stats, float* lse, int32_t nrec) {
+  __shared__ float2 red[LSE_THREADS / 32];
+  __shared__ float Ls;
+  pdl_launch_dependents();
+  pdl_wait();
+  const float L = row_lse(rec_stats + (int64_t)blockIdx.x * nrec, nrec, red, &Ls);
+  if (threadIdx.x == 0) lse[blockIdx.x] = L;
+}
+
+// CTA (chunk, row s), all rows of the last chunk first (the tiles written last
+// are still in L2: 258 us instead of 276 for the whole call at S = 272, V =
+// 128256): chunk of logits -> log-probabilities in place.  FUSED: every CTA of
+// row s also forms lse[s], one launch less (1.5 us at S = 9); otherwise
+// lm_lse_kernel has written it, so that a CTA's time is that of its loads and
+// stores alone (258 us instead of 266 at S = 272, equal at S = 65).
+template <bool FUSED, int CHUNK>
+__global__ void __launch_bounds__(LSE_THREADS) lm_lse_finalize_kernel(float* logits, const float2* rec_stats, float* lse,
+                                                                      int32_t S, int32_t V, int32_t nrec) {
+  const int tid = threadIdx.x, s = blockIdx.x % S, c = (gridDim.x - 1 - blockIdx.x) / S;
+  __shared__ float2 red[LSE_THREADS / 32];
+  __shared__ float Ls;
+  pdl_launch_dependents();
+  float* row = logits + (int64_t)s * V + (int64_t)c * CHUNK;
+  const int n = min(CHUNK, V - c * CHUNK);
+  float x[CHUNK / LSE_THREADS];
+  pdl_wait();
+#pragma unroll
+  for (int i = 0; i < CHUNK / LSE_THREADS; ++i)
+    if (tid + i * LSE_THREADS < n) x[i] = row[tid + i * LSE_THREADS];
+  float L;
+  if (FUSED) {
+    L = row_lse(rec_stats + (int64_t)s * nrec, nrec, red, &Ls);
+    if (c == 0 && tid == 0) lse[s] = L;
+  } else {
+    L = lse[s];
+  }
+#pragma unroll
+  for (int i = 0; i < CHUNK / LSE_THREADS; ++i)
+    if (tid + i * LSE_THREADS < n) row[tid + i * LSE_THREADS] = x[i] - L;
+}
+
+constexpr int LSE_FUSED_CHUNK = 8192;  // (144 CTAs for 9 rows of 128K entries)
+constexpr int LSE_CHUNK = 2048;
+
 cudaError_t lm_lse_finalize_launch(float* logits, const float2* rec_stats, float* lse, int32_t S, int32_t V,
-                                   int32_t nrec, cudaStream_t stream) {
-  lm_lse_finalize_kernel<<<dim3((V + LSE_CHUNK - 1) / LSE_CHUNK, S), 256, 0, stream>>>(logits, rec_stats, lse, V,
-                                                                                      nrec);
-  return cudaGetLastError();
+                                   int32_t nrec, bool fused, bool pdl, cudaStream_t stream) {
+  const int chunk = fused ? LSE_FUSED_CHUNK : LSE_CHUNK;
+  const dim3 grid((unsigned)((V + chunk - 1) / chunk) * (unsigned)S);
+  using pced_host::launch_kernel;
+  if (fused)
+    return launch_kernel(lm_lse_finalize_kernel<true, LSE_FUSED_CHUNK>, grid, LSE_THREADS, 0, stream, pdl, logits,
+                         rec_stats, lse, S, V, nrec);
+  const cudaError_t e = launch_kernel(lm_lse_kernel, dim3(S), LSE_THREADS, 0, stream, pdl, rec_stats, lse, nrec);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(lm_lse_finalize_kernel<false, LSE_CHUNK>, grid, LSE_THREADS, 0, stream, pdl, logits, rec_stats,
+                       lse, S, V, nrec);
 }
 
 // ------------------------------------------- Eq. 2 + Eq. 3 from tile records
@@ -734,7 +776,7 @@ extern "C" pced_status pced_lm_head_logprobs(const void* hidden, const void* w_u
   if (e != cudaSuccess) return cuda_status(e, "lm head tile counter");
   e = lm_head_launch(maps, g, a, s);
   if (e != cudaSuccess) return cuda_status(e, "lm head launch");
-  e = lm_lse_finalize_launch(logprobs, a.rec_stats, lse, S, V, g.ntiles, s);
+  e = lm_lse_finalize_launch(logprobs, a.rec_stats, lse, S, V, g.ntiles, S <= 64, true, s);
   if (e != cudaSuccess) return cuda_status(e, "lse finalize launch");
   return PCED_OK;
 }

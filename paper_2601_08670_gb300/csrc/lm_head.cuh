@@ -52,9 +52,10 @@ pced_status lm_head_maps(const void* w_unembed, const void* hidden, const LmGeom
 LmArgs lm_args(const LmGeom& g);  // the geometry's fields; the others zero
 cudaError_t lm_head_launch(const LmMaps& m, const LmGeom& g, const LmArgs& a, cudaStream_t stream);
 cudaError_t lm_head_pair_launch(const LmMaps& m, const LmGeom& g, const LmArgs& a, cudaStream_t stream);
-// mode-0 finish: lse[s] from the tile records, logits -> log-probs in place
+// mode-0 finish: lse[s] from the tile records, logits -> log-probs in place, in
+// one launch (fused) or two (pdl: as programmatic dependents)
 cudaError_t lm_lse_finalize_launch(float* logits, const float2* rec_stats, float* lse, int32_t S, int32_t V,
-                                   int32_t nrec, cudaStream_t stream);
+                                   int32_t nrec, bool fused, bool pdl, cudaStream_t stream);
 
 // Selection from mode-1 records (Eq. 2 + Eq. 3), one CTA per query.
 struct SelectArgs {

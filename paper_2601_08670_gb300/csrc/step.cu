@@ -324,7 +324,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     // needs the normalised rows
     if (e == cudaSuccess && dyn) {
       ranges.next("lse_finalize");
-      e = lm_lse_finalize_launch(W.lp, W.lm_stats, W.sel_L, S, dm.V, g.ntiles, s);
+      e = lm_lse_finalize_launch(W.lp, W.lm_stats, W.sel_L, S, dm.V, g.ntiles, true, !timed, s);
       if (e == cudaSuccess) e = mark();
     }
     // the JSD kernel also re-arms the LM head's tile counter for the fused pass
