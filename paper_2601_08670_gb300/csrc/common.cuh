@@ -527,20 +527,31 @@ pced_status make_tmap_kv(CUtensorMap* map, const void* base, uint64_t rows, uint
 // kernel.  Every kernel launched so calls pdl_wait() in all of its threads
 // before it touches memory that an earlier launch may write or still read, so
 // only its launch, and what it does before the wait, overlap that kernel.
-template <typename... P, typename... A>
-cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, bool pdl,
-                          A... args) {
+template <typename... P>
+cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int cluster, unsigned threads, size_t smem,
+                           cudaStream_t stream, bool pdl, P... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  if (pdl) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 0) {  // 0: as the kernel itself declares
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs++].val.clusterDim = {(unsigned)cluster, 1, 1};
+  }
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, bool pdl,
+                          A... args) {
+  return launch_cluster<P...>(kernel, grid, 0, threads, smem, stream, pdl, args...);
 }
 
 template <typename... P, typename... A>

@@ -19,6 +19,7 @@
 // Because shat_k(v) = u_k(v) + c_k with c_k = -(1+beta_k) L_k + beta_k L_0 + gamma log r_k
 // constant in v, Eq. 3 only needs these per-tile maxima and the log-sum-exps L:
 // the [S x V] logits never reach HBM on the fused path.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <stdlib.h>
 
@@ -27,6 +28,8 @@
 #include "select_key.cuh"
 
 namespace pced {
+
+namespace cg = cooperative_groups;
 
 constexpr int LM_PAIR_HSTAGES = 4;  // most stages of a pair's H ring
 
@@ -485,109 +488,136 @@ cudaError_t lm_lse_finalize_launch(float* logits, const float2* rec_stats, float
 }
 
 // ------------------------------------------- Eq. 2 + Eq. 3 from tile records
-// One CTA per row s = b*(N+1) + j: L_s from the row's tile records and, for an
-// expert row (j > 0), the best tile record of u_k; the last CTA of query b to
-// finish forms score_k = u_k* + c_k and picks the best (score desc, token
-// asc, expert asc).  Every reduction runs in a fixed order (thread t takes
-// records t, t + 256, ... in four interleaved chains, then a fixed tree), so
-// the result does not depend on timing.
-constexpr int SEL_R_THREADS = 256;
-constexpr int SEL_ZROWS = 12;  // hidden rows per block of the near-tie dot products
-
-__device__ __forceinline__ void lse_block(const float2* rec, int T, int tid, float2* red, float& L) {
-  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, su[4] = {0.f, 0.f, 0.f, 0.f};
-  int t = tid;
-  for (; t + 3 * SEL_R_THREADS < T; t += 4 * SEL_R_THREADS) {
-    float2 r[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) r[k] = rec[t + k * SEL_R_THREADS];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) lse_merge(m[k], su[k], r[k].x, r[k].y);
-  }
-  for (; t < T; t += SEL_R_THREADS) {
-    const float2 r = rec[t];
-    lse_merge(m[0], su[0], r.x, r.y);
-  }
-#pragma unroll
-  for (int k = 1; k < 4; ++k) lse_merge(m[0], su[0], m[k], su[k]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m[0], o), s2 = __shfl_xor_sync(0xffffffffu, su[0], o);
-    lse_merge(m[0], su[0], m2, s2);
-  }
-  if ((tid & 31) == 0) red[tid >> 5] = make_float2(m[0], su[0]);
-  __syncthreads();
-  if (tid == 0) {
-    float M = -INFINITY, Sm = 0.f;
-    for (int w = 0; w < SEL_R_THREADS / 32; ++w) lse_merge(M, Sm, red[w].x, red[w].y);
-    L = M + logf(Sm);
-  }
-}
+// One cluster of up to SEL_CLUSTER CTAs per query b; CTA c takes the rows j = c,
+// c + CTAs, ... of the query: L_s from the row's tile records and, for an
+// expert row (j > 0), the best tile record of u_k.  Every CTA gets every row's
+// results and forms score_k = u_k* + c_k and the pick (score desc, token asc,
+// expert asc); for the near-tie margins each recomputes z_s(token) of its own
+// rows, and the first one finishes.  Every reduction runs in a fixed order (a
+// row's threads take its records in turn, then xor trees over lanes, then the
+// warps in order), so the result does not depend on timing.
+//
+// What bounds it: a chain of dependent steps (records, the rows' exchange, the
+// chosen row of W, the exchange of the margins' products), all of latency.
+// The exchanges go through shared memory of the cluster, without the fences,
+// the arrival counter and the reloads of results in global memory that CTAs
+// without a cluster need, and the recomputed products, 129 rows of H at 128
+// experts, are spread over the cluster instead of one CTA.  A row's records are
+// in flight together and their maximum is the thread's own first, so one pass
+// does.  Measured (one CTA per row with an arrival counter -> this): 9 rows
+// 12.4 -> 10.1 us, 33 rows 17.4 -> 10.6, 129 rows 35 -> 21, 16 x 17 rows 19.0 ->
+// 13.2, 3 rows of d = 512 9.3 -> 8.4.
+constexpr int SEL_R_THREADS = 512;
+constexpr int SEL_R_WARPS = SEL_R_THREADS / 32;
+constexpr int SEL_R_CLUSTER = 8;  // most CTAs per query
+constexpr int SEL_RECS = 8;       // records of a thread in flight
+constexpr int SEL_ZROWS = 8;      // rows of a thread group in flight in the near-tie products
 
 __global__ void __launch_bounds__(SEL_R_THREADS) select_from_records_kernel(SelectArgs a) {
-  const int j = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int N = a.N, n1 = N + 1, s = b * n1 + j, T = a.nrec;
-  if (!PCED_IN_BOUNDS(s < a.B * n1, a.status)) return;
-  if (a.pdl) pdl_wait();  // the LM head's records are complete and visible
-  if (j == 0 && b == 0 && tid == 0 && a.tile_ctr) *a.tile_ctr = 0;  // the next LM head claims its tiles from 0
-  __shared__ float2 red[SEL_R_THREADS / 32];
-  __shared__ float sv[SEL_R_THREADS / 32], sv2[SEL_R_THREADS / 32];
-  __shared__ int si[SEL_R_THREADS / 32];
-  __shared__ int last;
-  __shared__ int pick[2];   // token, expert of the query (last CTA)
-  __shared__ float zy[LM_MAX_N1];  // z_s(token) of the query's rows (last CTA)
-  __shared__ float zpart[SEL_R_THREADS / 32][SEL_ZROWS];
-  float L = 0.f;
-  lse_block(a.rec_stats + (int64_t)s * T, T, tid, red, L);
-  if (j > 0) {
-    // the row's best u_k and its token, and the best u_k at any other token
-    const float2* rec = a.rec_arg + (int64_t)s * T;
-    const float* rec2 = a.rec_u2 + (int64_t)s * T;
-    float bu = -INFINITY, b2 = -INFINITY;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int nc = gridDim.x, rank = blockIdx.x, b = blockIdx.y;  // one cluster per query
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int N = a.N, n1 = N + 1, T = a.nrec;
+  __shared__ float row_L[LM_MAX_N1], row_u[LM_MAX_N1], row_u2[LM_MAX_N1];  // every row's results
+  __shared__ int row_tok[LM_MAX_N1];
+  __shared__ float zy[LM_MAX_N1];  // z_s(token) of the query's rows (first CTA)
+  __shared__ float sm[SEL_R_WARPS], su[SEL_R_WARPS], sv[SEL_R_WARPS], sv2[SEL_R_WARPS];
+  __shared__ int si[SEL_R_WARPS];
+  __shared__ int pick[2];  // token, expert of the query
+  __shared__ float zpart[SEL_R_WARPS][SEL_ZROWS];
+  cluster.barrier_arrive();  // waited for before another CTA's shared memory is written
+  if (a.pdl) pdl_wait();     // the LM head's records are complete and visible
+  if (rank == 0 && b == 0 && tid == 0 && a.tile_ctr) *a.tile_ctr = 0;  // the next LM head claims its tiles from 0
+  const int t_step = a.step && tid == 0 ? *a.step : 0;  // advances only once every query is through
+  // ---- the CTA's rows, rf at a time, SEL_R_WARPS / rf warps each
+  const int rows = (n1 - rank + nc - 1) / nc;
+  int rf = 1;
+  while (rf < rows && rf < 8) rf <<= 1;
+  const int wpr = SEL_R_WARPS / rf, grp = warp / wpr, gt = tid - grp * wpr * 32, gn = wpr * 32;
+  bool started = false;
+  for (int q0 = 0; q0 < rows; q0 += rf) {
+    const int q = q0 + grp, j = rank + nc * q, s = b * n1 + j;
+    const bool on = q < rows && PCED_IN_BOUNDS(s < a.B * n1, a.status);
+    // the row's (largest logit, sum of exp), its best u_k and its token, and the best u_k at any other token
+    float m = -INFINITY, sum = 0.f, bu = -INFINITY, b2 = -INFINITY;
     int bv = 0x7fffffff;
-    for (int t = tid; t < T; t += SEL_R_THREADS) {
-      const float2 r = rec[t];
-      top2_merge(bu, bv, b2, r.x, __float_as_int(r.y), rec2[t]);
-    }
+    if (on) {
+      const float2* rec = a.rec_stats + (int64_t)s * T;
+      const float2* reca = a.rec_arg + (int64_t)s * T;
+      const float* rec2 = a.rec_u2 + (int64_t)s * T;
+      for (int t0 = gt; t0 < T; t0 += SEL_RECS * gn) {
+        float2 st[SEL_RECS], ar[SEL_RECS];
+        float u2[SEL_RECS];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float r1 = __shfl_xor_sync(0xffffffffu, bu, o), r2 = __shfl_xor_sync(0xffffffffu, b2, o);
-      const int rt = __shfl_xor_sync(0xffffffffu, bv, o);
-      top2_merge(bu, bv, b2, r1, rt, r2);
+        for (int i = 0; i < SEL_RECS; ++i) {
+          const int t = t0 + i * gn;
+          const bool in = t < T;
+          st[i] = in ? __ldcg(rec + t) : make_float2(-INFINITY, 0.f);
+          ar[i] = in && j > 0 ? __ldcg(reca + t) : make_float2(-INFINITY, __int_as_float(0x7fffffff));
+          u2[i] = in && j > 0 ? __ldcg(rec2 + t) : -INFINITY;
+        }
+        float mn = m;
+#pragma unroll
+        for (int i = 0; i < SEL_RECS; ++i) mn = fmaxf(mn, st[i].x);
+        if (m != -INFINITY) sum *= expf(m - mn);
+#pragma unroll
+        for (int i = 0; i < SEL_RECS; ++i) {
+          if (st[i].x != -INFINITY) sum += st[i].y * expf(st[i].x - mn);
+          top2_merge(bu, bv, b2, ar[i].x, __float_as_int(ar[i].y), u2[i]);
+        }
+        m = mn;
+      }
+      const float mw = warp_max(m);
+      sum = warp_sum(m == -INFINITY ? sum : sum * expf(m - mw));
+      m = mw;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float r1 = __shfl_xor_sync(0xffffffffu, bu, o), r2 = __shfl_xor_sync(0xffffffffu, b2, o);
+        const int rt = __shfl_xor_sync(0xffffffffu, bv, o);
+        top2_merge(bu, bv, b2, r1, rt, r2);
+      }
     }
     if (lane == 0) {
+      sm[warp] = m;
+      su[warp] = sum;
       sv[warp] = bu;
       si[warp] = bv;
       sv2[warp] = b2;
     }
     __syncthreads();
-    if (tid == 0) {
-      for (int w = 1; w < SEL_R_THREADS / 32; ++w) top2_merge(bu, bv, b2, sv[w], si[w], sv2[w]);
-      a.sel_u[s] = bu;
-      a.sel_tok[s] = bv;
-      a.sel_u2[s] = b2;
+    if (!started) cluster.barrier_wait();
+    started = true;
+    if (on && gt < nc) {  // thread gt writes the row's results to CTA gt
+      float M = -INFINITY, L = 0.f;
+      bu = b2 = -INFINITY;
+      bv = 0x7fffffff;
+      for (int w = grp * wpr; w < (grp + 1) * wpr; ++w) {
+        M = fmaxf(M, sm[w]);
+        top2_merge(bu, bv, b2, sv[w], si[w], sv2[w]);
+      }
+      for (int w = grp * wpr; w < (grp + 1) * wpr; ++w) L += sm[w] == -INFINITY ? su[w] : su[w] * expf(sm[w] - M);
+      L = M + logf(L);
+      cluster.map_shared_rank(row_L, gt)[j] = L;
+      cluster.map_shared_rank(row_u, gt)[j] = bu;
+      cluster.map_shared_rank(row_u2, gt)[j] = b2;
+      cluster.map_shared_rank(row_tok, gt)[j] = bv;
+      if (gt == 0 && a.lse_out) a.lse_out[s] = L;
     }
+    if (q0 + rf < rows) __syncthreads();  // the partial results are used again
   }
-  if (tid == 0) {
-    a.sel_L[s] = L;
-    if (a.lse_out) a.lse_out[s] = L;
-    __threadfence();
-    last = atomicAdd(a.qdone + b, 1) == n1 - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();  // the other rows' results of query b are visible
-  const float L0 = __ldcg(a.sel_L + b * n1);
+  cluster.sync();
   float bs = -INFINITY;
   int bt = 0x7fffffff, bk = 0x7fffffff;
+  // Eq. 2's per-expert constant
+  auto bias = [&](int k) {
+    const float btk = a.beta[b * N + k];
+    const float rr = fminf(fmaxf(a.r[b * N + k], 1e-8f), 1.0f);
+    return (a.raw_logits ? 0.f : -(1.f + btk) * row_L[1 + k] + btk * row_L[0]) + a.gamma * logf(rr);
+  };
   if (warp == 0) {
     for (int k = lane; k < N; k += 32) {
-      const int sk = b * n1 + 1 + k;
-      const float btk = a.beta[b * N + k];
-      const float rr = fminf(fmaxf(a.r[b * N + k], 1e-8f), 1.0f);
-      const float c = (a.raw_logits ? 0.f : -(1.f + btk) * __ldcg(a.sel_L + sk) + btk * L0) + a.gamma * logf(rr);
-      const float sc = __ldcg(a.sel_u + sk) + c;
-      const int tk = __ldcg(a.sel_tok + sk);
+      const float sc = row_u[1 + k] + bias(k);
+      const int tk = row_tok[1 + k];
       if (sc > bs || (sc == bs && (tk < bt || (tk == bt && k < bk)))) {
         bs = sc;
         bt = tk;
@@ -613,70 +643,62 @@ __global__ void __launch_bounds__(SEL_R_THREADS) select_from_records_kernel(Sele
   if (a.gap_trace && !a.key_out) {
     __syncthreads();
     const int y = pick[0] >= 0 && pick[0] < a.V ? pick[0] : 0;
-    // z_s(y) = h_s . W[y] for the query's rows.  Thread t takes the 16-byte
-    // chunks i = t, t + 256 of W[y] and the same chunks of up to 16 rows at a
-    // time, all loads of a row block in flight together (one round trip for
-    // d <= 4096); per row the partial sums meet in a fixed order (warp tree,
-    // then the warps in order).
+    // z_s(y) = h_s . W[y] for the CTA's rows.  tpr threads take a row (16-byte
+    // chunks i, i + tpr, ... of W[y] and of the row), SEL_ZROWS rows of each
+    // group of tpr threads in flight together.  Per row the partial sums meet
+    // in a fixed order (warp tree, then the group's warps in order).
     const int nv = a.d / 8;  // 16-byte chunks of a row (d % 64 == 0)
+    int tpr = 32;
+    while (tpr < nv && tpr < SEL_R_THREADS / (rows > 1 ? 2 : 1)) tpr <<= 1;
+    const int ng = SEL_R_THREADS / tpr, g = tid / tpr, wpg = tpr / 32;
     const uint4* wy = reinterpret_cast<const uint4*>(a.w_unembed + (int64_t)y * a.d);
     const uint4* h0 = reinterpret_cast<const uint4*>(a.hidden + (int64_t)b * n1 * a.d);
-    for (int r0 = 0; r0 < n1; r0 += SEL_ZROWS) {
+    for (int q0 = 0; q0 < rows; q0 += ng * SEL_ZROWS) {
       float acc[SEL_ZROWS];
 #pragma unroll
-      for (int r = 0; r < SEL_ZROWS; ++r) acc[r] = 0.f;
-      for (int i0 = tid; i0 < nv; i0 += 2 * SEL_R_THREADS) {
-        uint4 wv[2], hv[2][SEL_ZROWS];
+      for (int u = 0; u < SEL_ZROWS; ++u) acc[u] = 0.f;
+      for (int i = tid % tpr; i < nv; i += tpr) {
+        const uint4 wv = __ldg(wy + i);
+        uint4 hv[SEL_ZROWS];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int i = i0 + u * SEL_R_THREADS;
-          if (i < nv) wv[u] = __ldg(wy + i);
-#pragma unroll
-          for (int r = 0; r < SEL_ZROWS; ++r)
-            if (i < nv && r0 + r < n1) hv[u][r] = __ldcg(h0 + (int64_t)(r0 + r) * nv + i);
+        for (int u = 0; u < SEL_ZROWS; ++u) {
+          const int q = q0 + g + ng * u;
+          hv[u] = q < rows ? __ldcg(h0 + (int64_t)(rank + nc * q) * nv + i) : make_uint4(0u, 0u, 0u, 0u);
         }
+        const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (i0 + u * SEL_R_THREADS >= nv) continue;
-          const uint32_t ww[4] = {wv[u].x, wv[u].y, wv[u].z, wv[u].w};
+        for (int u = 0; u < SEL_ZROWS; ++u) {
+          const uint32_t hw[4] = {hv[u].x, hv[u].y, hv[u].z, hv[u].w};
+          float p = 0.f;
 #pragma unroll
-          for (int r = 0; r < SEL_ZROWS; ++r) {
-            if (r0 + r >= n1) continue;
-            const uint32_t hw[4] = {hv[u][r].x, hv[u][r].y, hv[u][r].z, hv[u][r].w};
-            float p = 0.f;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              p = fmaf(bf16_lo(hw[q]), bf16_lo(ww[q]), p);
-              p = fmaf(bf16_hi(hw[q]), bf16_hi(ww[q]), p);
-            }
-            acc[r] += p;
+          for (int e = 0; e < 4; ++e) {
+            p = fmaf(bf16_lo(hw[e]), bf16_lo(ww[e]), p);
+            p = fmaf(bf16_hi(hw[e]), bf16_hi(ww[e]), p);
           }
+          acc[u] += p;
         }
       }
 #pragma unroll
-      for (int r = 0; r < SEL_ZROWS; ++r) {
-        const float t = warp_sum(acc[r]);
-        if (lane == 0) zpart[warp][r] = t;
+      for (int u = 0; u < SEL_ZROWS; ++u) {
+        const float t = warp_sum(acc[u]);
+        if (lane == 0) zpart[warp][u] = t;
       }
       __syncthreads();
-      if (tid < SEL_ZROWS && r0 + tid < n1) {
+      if (tid < ng * SEL_ZROWS && q0 + tid < rows) {
+        // row q0 + tid of the CTA: group tid % ng, slot tid / ng
         float z = 0.f;
-        for (int w = 0; w < SEL_R_THREADS / 32; ++w) z += zpart[w][tid];
-        zy[r0 + tid] = z;
+        for (int w = 0; w < wpg; ++w) z += zpart[(tid % ng) * wpg + w][tid / ng];
+        cluster.map_shared_rank(zy, 0)[rank + nc * (q0 + tid)] = z;
       }
       __syncthreads();
     }
-    if (warp == 0) {
+    cluster.sync();
+    if (warp == 0 && rank == 0) {
       // token gap: the best score at another token, over all experts
       float other = -INFINITY, se_best = -INFINITY, se_other = -INFINITY;
       for (int k = lane; k < N; k += 32) {
-        const int sk = b * n1 + 1 + k;
-        const float btk = a.beta[b * N + k];
-        const float rr = fminf(fmaxf(a.r[b * N + k], 1e-8f), 1.0f);
-        const float Lk = __ldcg(a.sel_L + sk);
-        const float c = (a.raw_logits ? 0.f : -(1.f + btk) * Lk + btk * L0) + a.gamma * logf(rr);
-        const float cand = __ldcg(a.sel_tok + sk) != bt ? __ldcg(a.sel_u + sk) : __ldcg(a.sel_u2 + sk);
-        other = fmaxf(other, cand + c);
+        const float c = bias(k), btk = a.beta[b * N + k];
+        other = fmaxf(other, (row_tok[1 + k] != bt ? row_u[1 + k] : row_u2[1 + k]) + c);
         // expert gap: every expert's score at the chosen token, from the recomputed logits
         const float se = (1.f + btk) * zy[1 + k] - btk * zy[0] + c;
         if (k == bk) se_best = se;
@@ -688,21 +710,20 @@ __global__ void __launch_bounds__(SEL_R_THREADS) select_from_records_kernel(Sele
       gaps = make_float2(bs - other, se_best - se_other);
     }
   }
+  if (rank != 0) return;
   if (warp != 0) return;
   if (lane == 0 && a.key_out) {
     // expert-partitioned step: this GPU's best, the reduction over GPUs and
     // the append come after
-    a.qdone[b] = 0;
     a.key_out[b] = select_key(bs, bt, a.expert_base + bk + 1);
     return;
   }
   if (lane == 0) {
-    a.qdone[b] = 0;
     if (a.token) a.token[b] = bt;
     if (a.expert) a.expert[b] = bk + 1;
     if (a.score) a.score[b] = bs;
     if (a.step) {
-      const int t = *a.step;
+      const int t = t_step;
       if (t >= 0 && t < a.max_steps) {
         a.history[(int64_t)b * a.max_steps + t] = bt;
         if (a.expert_trace) a.expert_trace[(int64_t)b * a.max_steps + t] = bk + 1;
@@ -711,27 +732,22 @@ __global__ void __launch_bounds__(SEL_R_THREADS) select_from_records_kernel(Sele
       } else {
         dev_flag(a.status, PCED_DEV_STEP_LIMIT);
       }
-      __threadfence();
-      if (atomicAdd(a.done_counter, 1) == a.B - 1) {
-        if (t >= 0 && t < a.max_steps) *a.step = t + 1;  // at the limit t stays (as the commit does)
-        *a.done_counter = 0;
+      bool all = a.B == 1;
+      if (!all) {
         __threadfence();
+        all = atomicAdd(a.done_counter, 1) == a.B - 1;
+        if (all) *a.done_counter = 0;
       }
+      if (all && t >= 0 && t < a.max_steps) *a.step = t + 1;  // at the limit t stays (as the commit does)
     }
   }
 }
 
 cudaError_t select_from_records_launch(const SelectArgs& a, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.N + 1, a.B);
-  cfg.blockDim = dim3(SEL_R_THREADS);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = a.pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, select_from_records_kernel, a);
+  int nc = 1;  // CTAs per query: a power of two, at most one per row
+  while (2 * nc <= SEL_R_CLUSTER && 2 * nc <= a.N + 1) nc *= 2;
+  return pced_host::launch_cluster(select_from_records_kernel, dim3(nc, a.B), nc, SEL_R_THREADS, 0, stream, a.pdl != 0,
+                                   a);
 }
 
 }  // namespace pced

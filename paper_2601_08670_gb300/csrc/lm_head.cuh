@@ -57,7 +57,7 @@ cudaError_t lm_head_pair_launch(const LmMaps& m, const LmGeom& g, const LmArgs& 
 cudaError_t lm_lse_finalize_launch(float* logits, const float2* rec_stats, float* lse, int32_t S, int32_t V,
                                    int32_t nrec, bool fused, bool pdl, cudaStream_t stream);
 
-// Selection from mode-1 records (Eq. 2 + Eq. 3), one CTA per query.
+// Selection from mode-1 records (Eq. 2 + Eq. 3), one cluster per query.
 struct SelectArgs {
   const float2* rec_stats;
   const float2* rec_arg;
@@ -79,12 +79,6 @@ struct SelectArgs {
   float* score_trace;
   int32_t max_steps;
   int32_t* done_counter;
-  // per-row results and per-query counters (zero at the first launch; the
-  // last CTA of a query resets its counter)
-  float* sel_L;       // [S] log-sum-exp of each row
-  float* sel_u;       // [S] best u_k of each expert row
-  int32_t* sel_tok;   // [S] its token
-  float* sel_u2;      // [S] the row's best u_k at another token
   // near-tie margins of the choice (optional): gap_trace[b][t] = (token gap,
   // expert gap); the expert gap recomputes z_s(y) = h_s . W[y] for the
   // query's rows
@@ -94,7 +88,6 @@ struct SelectArgs {
   const __nv_bfloat16* hidden;     // [S][d]
   const __nv_bfloat16* w_unembed;  // [V][d]
   int32_t d;
-  int32_t* qdone;     // [B] rows of the query finished
   int pdl;            // launched as a programmatic dependent of the LM head
   int raw_logits;     // s_k of Eq. 2 are the raw logits: c_k = gamma log r_k alone
   int* status;

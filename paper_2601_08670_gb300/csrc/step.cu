@@ -27,10 +27,7 @@ struct StepLayout {
   int32_t* att_done;      // attention: CTAs finished
   int32_t* att_epoch;     // attention: launches completed
   int32_t* lm_tile_ctr;   // LM head: vocabulary tiles claimed (reset by the selection)
-  int32_t* sel_qdone;     // selection: rows finished per query
-  float* sel_L;
-  float* sel_u;
-  int32_t* sel_tok;
+  float* sel_L;           // log-sum-exps of the rows (dynamic beta, MoE / PoE)
   float* lp;              // [S][V] log-probabilities of a dynamic-beta first step
   float2* agg_part;       // MoE / PoE: per (query, expert, chunk) statistics
   float2* agg_best;       // MoE / PoE: per (query, chunk) best
@@ -46,7 +43,6 @@ struct StepLayout {
   float2* lm_stats;
   float2* lm_arg;
   float* lm_u2;
-  float* sel_u2;
   size_t bytes;
 };
 
@@ -70,12 +66,8 @@ static StepLayout step_layout(const pced_dims* dm, void* ws) {
   L.lm_stats = c.take<float2>((size_t)(S * ntiles));
   L.lm_arg = c.take<float2>((size_t)(S * ntiles));
   L.lm_u2 = c.take<float>((size_t)(S * ntiles));
-  L.sel_u2 = c.take<float>((size_t)S);
   L.lm_tile_ctr = c.take<int32_t>(1);
-  L.sel_qdone = c.take<int32_t>((size_t)dm->B);
   L.sel_L = c.take<float>((size_t)S);
-  L.sel_u = c.take<float>((size_t)S);
-  L.sel_tok = c.take<int32_t>((size_t)S);
   L.lp = c.take<float>((size_t)S * dm->V);
   L.agg_part = c.take<float2>((size_t)dm->B * dm->N * agg_chunks(dm->V));
   L.agg_best = c.take<float2>((size_t)dm->B * agg_chunks(dm->V));
@@ -409,7 +401,6 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   sa.rec_arg = W.lm_arg;
   sa.rec_u2 = W.lm_u2;
   sa.V = dm.V;
-  sa.sel_u2 = W.sel_u2;
   sa.gap_trace = reinterpret_cast<float2*>(p->gap_trace);
   sa.key_out = p->key_out;
   sa.expert_base = p->expert_base;
@@ -420,10 +411,6 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   sa.N = dm.N;
   sa.nrec = g.ntiles;
   sa.tile_ctr = W.lm_tile_ctr;
-  sa.sel_L = W.sel_L;
-  sa.sel_u = W.sel_u;
-  sa.sel_tok = W.sel_tok;
-  sa.qdone = W.sel_qdone;
   sa.beta = beta;
   sa.r = p->r;
   sa.gamma = p->gamma;
