@@ -7,15 +7,15 @@
 //   beta[b][k-1] = 1/2 sum_v [ p_k log2(p_k / m) + p_0 log2(p_0 / m) ],  m = (p_k + p_0) / 2,
 // in [0, 1].  With hi / lo the larger and smaller of the two log-probabilities
 // and e = exp(lo - hi), a term is
-//   exp(hi) [ q + e (q + lo - hi) ],  q = ln 2 - log1p(e) = log(p_hi / m),
+//   exp(hi) [ q + e (q + lo - hi) ],  q = -log((1 + e) / 2) = log(p_hi / m),
 // in fp32, without the rounding of a logarithm of the size of hi.
 //
-// What bounds it: two exp and one log1p per entry and expert (and, past the
-// L2, the rows).  A cluster of ADA_CLUSTER CTAs takes one (expert, query): the
+// What bounds it: two exp and one log per entry and expert (and, past the
+// L2, the rows).  A cluster of CTAs takes one (expert, query): the
 // cluster's sums meet in the first CTA's shared memory, so there is no scratch,
 // no counter to clear and no second pass.  (One CTA per 2048 entries left the
 // last one to add 63 chunk sums one load after the other: 14.8 us for 8
-// experts of 128256 entries beside a memset; 180 us for 16 x 16.)
+// experts of 128256 entries beside a memset; 184 us for 16 x 16, now 86.)
 //
 // Sums are held as an unevaluated pair of fp32 numbers (error-free addition,
 // about 48 bits) and rounded once from fp64 at the end: this chip adds 64-bit
@@ -33,7 +33,6 @@ namespace pced {
 namespace cg = cooperative_groups;
 
 constexpr int ADA_THREADS = 1024;
-constexpr int ADA_CLUSTER = 8;
 constexpr int ADA_UNROLL = 4;  // entries of a thread in flight
 
 // an fp32 pair s + c, |c| below half an ulp of s times the terms added
@@ -65,26 +64,25 @@ __device__ __forceinline__ Pair warp_pair(Pair p) {
 }
 
 __device__ __forceinline__ float jsd_term(float a, float b) {
-  const float ln2 = 0.69314718055994531f;
   const float hi = fmaxf(a, b), lo = fminf(a, b);
   if (hi == -INFINITY) return 0.f;  // both probabilities are 0
-  const float d = lo - hi, e = expf(d), q = ln2 - log1pf(e);
+  const float d = lo - hi, e = expf(d), q = -logf(fmaf(0.5f, e, 0.5f));
   return expf(hi) * (lo == -INFINITY ? q : q + e * (q + d));
 }
 
-// grid (ADA_CLUSTER, N, B), one cluster per (k - 1, b)
-__global__ void __cluster_dims__(ADA_CLUSTER, 1, 1) __launch_bounds__(ADA_THREADS)
+// grid (CTAs of a cluster, N, B), one cluster per (k - 1, b)
+__global__ void __launch_bounds__(ADA_THREADS)
     adacad_beta_kernel(const float* __restrict__ lp, int32_t N, int32_t V, float* beta, int* reset_ctr) {
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = blockIdx.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
-  __shared__ Pair wsum[ADA_THREADS / 32], csum[ADA_CLUSTER];
+  const int rank = blockIdx.x, nc = gridDim.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
+  __shared__ Pair wsum[ADA_THREADS / 32], csum[ROW_CLUSTER];
   cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
   pdl_launch_dependents();
   pdl_wait();
   if (reset_ctr && rank == 0 && k == 1 && b == 0 && tid == 0) *reset_ctr = 0;
   const float* l0 = lp + (int64_t)b * (N + 1) * V;
   const float* lk = l0 + (int64_t)k * V;
-  const int per = (int)(((int64_t)V + ADA_CLUSTER - 1) / ADA_CLUSTER);
+  const int per = (V - 1) / nc + 1;
   const int64_t v0 = (int64_t)rank * per, v1 = min((int64_t)V, v0 + per);
   Pair acc{0.f, 0.f};
   for (int64_t v = v0 + tid; v < v1; v += ADA_UNROLL * ADA_THREADS) {
@@ -107,17 +105,16 @@ __global__ void __cluster_dims__(ADA_CLUSTER, 1, 1) __launch_bounds__(ADA_THREAD
   cluster.sync();
   if (rank == 0 && tid == 0) {
     Pair t = csum[0];
-    for (int i = 1; i < ADA_CLUSTER; ++i) t = pair_merge(t, csum[i]);
+    for (int i = 1; i < nc; ++i) t = pair_merge(t, csum[i]);
     beta[(int64_t)b * N + k - 1] = (float)(((double)t.s + (double)t.c) * 0.72134752044448170);  // 1 / (2 ln 2)
   }
 }
 
 cudaError_t adacad_beta_launch(const float* lp, int32_t B, int32_t N, int32_t V, float* beta, int* reset_ctr, bool pdl,
                                cudaStream_t stream) {
-  const dim3 grid(ADA_CLUSTER, N, B);
-  if (pdl) return pced_host::launch_pdl(adacad_beta_kernel, grid, ADA_THREADS, 0, stream, lp, N, V, beta, reset_ctr);
-  adacad_beta_kernel<<<grid, ADA_THREADS, 0, stream>>>(lp, N, V, beta, reset_ctr);
-  return cudaGetLastError();
+  const int nc = pced_host::row_cluster((int64_t)B * N);
+  return pced_host::launch_cluster(adacad_beta_kernel, dim3(nc, N, B), nc, ADA_THREADS, 0, stream, pdl, lp, N, V, beta,
+                                   reset_ctr);
 }
 
 }  // namespace pced

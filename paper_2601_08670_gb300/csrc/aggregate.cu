@@ -7,13 +7,21 @@
 //   MoE: agg(v) = log sum_k w_k p_k(v)     PoE: agg(v) = sum_k w_k log p_k(v)
 //   token = argmax_v agg (lowest id on ties), score = agg(token),
 //   expert = argmax_k w_k p_k(token) (lowest k on ties).
-// Two launches over the materialised log-probabilities (S x V fp32, a few MB,
-// L2-resident): (1) per (query, expert, chunk) the max and sum of exp of c_k,
-// merged into the expert's log-sum-exp by the last chunk to finish; (2) per
+// Two launches over the materialised log-probabilities (S x V fp32): (1) a
+// cluster of CTAs per (query, expert) forms the log-sum-exp of c_k; (2) per
 // (query, chunk) the best aggregate and the best at another token; the last
 // CTA of a query picks the token across chunks, attributes the expert and
 // writes the step's results with both near-tie margins.  Every sum runs in a
 // fixed order, so results do not depend on timing.
+//
+// What bounds them: latency for one query (a few MB in L2), the rows' bytes
+// and one exp per entry and kernel for many.  (1) with a CTA, a fence and an
+// arrival per 1024 entries and two exps per entry: 11-12 us for 8 experts of
+// 128256 entries, 151 us for 16 x 16.  A thread now has AGG_UNROLL entries in
+// flight and scales once per batch, and the cluster's sums meet in shared
+// memory: 8.4 and 59 us.  (2) with one load in flight per thread: 13 and 65 us;
+// with four tokens of four experts 9.4 and 37 us.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "aggregate.cuh"
@@ -21,7 +29,12 @@
 
 namespace pced {
 
-constexpr int AGG_THREADS = 256;
+namespace cg = cooperative_groups;
+
+constexpr int AGG_THREADS = 256;     // selection kernel
+constexpr int AGG_L_THREADS = 1024;  // log-sum-exp kernel
+constexpr int AGG_UNROLL = 8;        // entries of a thread in flight (log-sum-exp kernel)
+constexpr int AGG_TOK = AGG_CHUNK / AGG_THREADS, AGG_ROWS = 4;  // tokens and expert rows in flight (selection)
 
 __device__ __forceinline__ void agg_lse_merge(float& m, float& s, float m2, float s2) {
   if (m2 == -INFINITY) return;
@@ -35,70 +48,85 @@ __device__ __forceinline__ void agg_lse_merge(float& m, float& s, float m2, floa
   m = M;
 }
 
-// grid (nchunks, N, B): the chunk's (max, sum exp) of c_k; the last chunk CTA
-// of (query, expert) to finish merges them all into lse_k (strided, then a
-// fixed tree: the order does not depend on which CTA is last)
-__global__ void __launch_bounds__(AGG_THREADS) agg_partials_kernel(AggArgs a) {
-  const int c = blockIdx.x, k = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+// log-sum-exp over a warp of per-lane (m, s)
+__device__ __forceinline__ void warp_lse(float& m, float& s) {
+  const float M = warp_max(m);
+  s = warp_sum(m == -INFINITY ? s : s * expf(m - M));
+  m = M;
+}
+
+// (m, s) over the CTA's threads, in thread 0
+__device__ __forceinline__ void block_lse(float& m, float& s, float2* red) {
+  const int tid = threadIdx.x;
+  warp_lse(m, s);
+  __syncthreads();
+  if ((tid & 31) == 0) red[tid >> 5] = make_float2(m, s);
+  __syncthreads();
+  if (tid < 32) {
+    m = red[tid].x;
+    s = red[tid].y;
+    warp_lse(m, s);
+  }
+}
+
+// grid (CTAs of a cluster, N, B): lse_k of (query b, expert k); with rec_stats also
+// the rows' own log-sum-exps
+__global__ void __launch_bounds__(AGG_L_THREADS) agg_partials_kernel(AggArgs a) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = blockIdx.x, nc = gridDim.x, k = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
   const int N = a.N, V = a.V;
+  __shared__ float2 red[AGG_L_THREADS / 32], part[ROW_CLUSTER];
+  cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
+  pdl_launch_dependents();
+  pdl_wait();
   const float* lp0 = a.lp + (int64_t)b * (N + 1) * V;
   const float* lpk = lp0 + (int64_t)(k + 1) * V;
   const float bt = a.beta[b * N + k];
-  __shared__ float2 red[AGG_THREADS / 32];
-  __shared__ int last;
-  auto block_merge = [&](float m, float s) -> float2 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
-      agg_lse_merge(m, s, m2, s2);
-    }
-    if ((tid & 31) == 0) red[tid >> 5] = make_float2(m, s);
-    __syncthreads();
-    float M = -INFINITY, Sm = 0.f;
-    for (int w = 0; w < AGG_THREADS / 32; ++w) agg_lse_merge(M, Sm, red[w].x, red[w].y);
-    __syncthreads();
-    return make_float2(M, Sm);
-  };
-  if (a.rec_stats && c == 0) {
-    // raw logits: the log-sum-exps of expert k's row (and, for k = 0, the
-    // amateur's) from the LM head's tile records, in a fixed order
-    for (int r = 0; r < (k == 0 ? 2 : 1); ++r) {
-      const int64_t row = (int64_t)b * (N + 1) + (r == 0 ? k + 1 : 0);
-      float mm = -INFINITY, ss = 0.f;
-      for (int j = tid; j < a.nrec; j += AGG_THREADS) {
-        const float2 e = a.rec_stats[row * a.nrec + j];
-        agg_lse_merge(mm, ss, e.x, e.y);
-      }
-      const float2 t = block_merge(mm, ss);
-      if (tid == 0) a.lse_rows[row] = t.x + logf(t.y);
-    }
-  }
+  const int per = (V - 1) / nc + 1;
+  const int64_t v0 = (int64_t)rank * per, v1 = min((int64_t)V, v0 + per);
   float m = -INFINITY, s = 0.f;
-  const int v1 = min(V, (c + 1) * AGG_CHUNK);
-  for (int v = c * AGG_CHUNK + tid; v < v1; v += AGG_THREADS) {
-    const float ck = (1.f + bt) * lpk[v] - bt * lp0[v];
-    agg_lse_merge(m, s, ck, 1.f);
+  for (int64_t v = v0 + tid; v < v1; v += AGG_UNROLL * AGG_L_THREADS) {
+    float x[AGG_UNROLL], y[AGG_UNROLL];
+#pragma unroll
+    for (int u = 0; u < AGG_UNROLL; ++u) {
+      const bool in = v + u * AGG_L_THREADS < v1;
+      x[u] = in ? lpk[v + u * AGG_L_THREADS] : -INFINITY;
+      y[u] = in ? lp0[v + u * AGG_L_THREADS] : 0.f;
+    }
+    float mn = m;
+#pragma unroll
+    for (int u = 0; u < AGG_UNROLL; ++u) {
+      x[u] = (1.f + bt) * x[u] - bt * y[u];
+      if (v + u * AGG_L_THREADS >= v1) x[u] = -INFINITY;  // whatever beta is
+      mn = fmaxf(mn, x[u]);
+    }
+    if (m != -INFINITY) s *= expf(m - mn);
+    m = mn;
+#pragma unroll
+    for (int u = 0; u < AGG_UNROLL; ++u)
+      if (x[u] != -INFINITY) s += expf(x[u] - m);
   }
-  const float2 ms = block_merge(m, s);
-  const int64_t pk = (int64_t)b * N + k;
-  if (tid == 0) {
-    a.part[pk * a.nchunks + c] = ms;
-    __threadfence();
-    last = atomicAdd(a.kdone + pk, 1) == a.nchunks - 1;
+  block_lse(m, s, red);
+  cluster.barrier_wait();
+  if (tid == 0) *cluster.map_shared_rank(part + rank, 0) = make_float2(m, s);
+  cluster.sync();
+  if (rank == 0 && tid == 0) {
+    for (int i = 1; i < nc; ++i) agg_lse_merge(m, s, part[i].x, part[i].y);
+    a.lse_k[(int64_t)b * N + k] = m + logf(s);
   }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();  // the other chunks' statistics are visible
-  m = -INFINITY;
-  s = 0.f;
-  for (int j = tid; j < a.nchunks; j += AGG_THREADS) {
-    const float2 e = __ldcg(a.part + pk * a.nchunks + j);
-    agg_lse_merge(m, s, e.x, e.y);
-  }
-  const float2 t = block_merge(m, s);
-  if (tid == 0) {
-    a.lse_k[pk] = t.x + logf(t.y);
-    a.kdone[pk] = 0;
+  // raw logits: the log-sum-exps of expert k's row and, for k = 0, the amateur's
+  // (by other CTAs where there are some) from the LM head's tile records, in a fixed order
+  for (int i = 0; a.rec_stats && i < (k == 0 ? 2 : 1); ++i) {
+    if (rank != (i + 1) % nc) continue;
+    const int64_t row = (int64_t)b * (N + 1) + (i == 0 ? k + 1 : 0);
+    m = -INFINITY;
+    s = 0.f;
+    for (int j = tid; j < a.nrec; j += AGG_L_THREADS) {
+      const float2 e = a.rec_stats[row * a.nrec + j];
+      agg_lse_merge(m, s, e.x, e.y);
+    }
+    block_lse(m, s, red);
+    if (tid == 0) a.lse_rows[row] = m + logf(s);
   }
 }
 
@@ -121,55 +149,84 @@ __device__ __forceinline__ void agg_top2(float& b1, int& t1, float& b2, float r1
 // log-probabilities: per token the best expert's score of Eq. 2 (the first
 // step of a dynamic-beta decode selects this way, from the log-probabilities
 // it has written for beta anyway); rules 1 and 2 are MoE and PoE.
+template <int RULE>
 __global__ void __launch_bounds__(AGG_THREADS) agg_select_kernel(AggArgs a) {
   const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = a.N, V = a.V, n1 = N + 1;
-  __shared__ float w_s[AGG_MAX_N], lse_s[AGG_MAX_N], beta_s[AGG_MAX_N];
-  __shared__ float wsum;
+  // w_s: r clipped; wn_s: normalised weights; lse_s: per-expert constants
+  __shared__ float w_s[AGG_MAX_N], wn_s[AGG_MAX_N], lse_s[AGG_MAX_N], beta_s[AGG_MAX_N];
+  __shared__ float wsum[AGG_THREADS / 32];
   __shared__ float bv_s[AGG_THREADS / 32], b2_s[AGG_THREADS / 32];
   __shared__ int bt_s[AGG_THREADS / 32];
   __shared__ int last;
+  pdl_wait();
   if (c == 0 && b == 0 && tid == 0 && a.tile_ctr) *a.tile_ctr = 0;  // the next LM head claims its tiles from 0
+  const float* lp0 = a.lp + (int64_t)b * n1 * V;
+  const int v0 = c * AGG_CHUNK + tid;
+  float l0[AGG_TOK], acc[AGG_TOK];
+#pragma unroll
+  for (int j = 0; j < AGG_TOK; ++j) {
+    l0[j] = v0 + j * AGG_THREADS < V ? lp0[v0 + j * AGG_THREADS] : 0.f;
+    acc[j] = RULE == 0 ? -INFINITY : 0.f;
+  }
+  float t = 0.f;
   for (int k = tid; k < N; k += AGG_THREADS) {
-    w_s[k] = fminf(fmaxf(a.r[b * N + k], 1e-8f), 1.0f);
+    const float w = fminf(fmaxf(a.r[b * N + k], 1e-8f), 1.0f);
+    w_s[k] = w;
+    t += w;
     beta_s[k] = a.beta[b * N + k];
-    if (a.rule == 0) {
+    if (RULE == 0) {
       // the per-expert constant of Eq. 2: gamma log r_k (plus the log-sum-exps
       // when s_k are raw logits: z = lp + L)
       const float btk = beta_s[k];
-      lse_s[k] = a.gamma * logf(w_s[k]) +
-                 (a.raw_logits ? (1.f + btk) * a.lse[b * n1 + 1 + k] - btk * a.lse[b * n1] : 0.f);
+      lse_s[k] = a.gamma * logf(w) + (a.raw_logits ? (1.f + btk) * a.lse[b * n1 + 1 + k] - btk * a.lse[b * n1] : 0.f);
     } else {
       lse_s[k] = a.lse_k[(int64_t)b * N + k];
     }
   }
-  __syncthreads();
-  if (tid == 0) {
-    float t = 0.f;
-    for (int k = 0; k < N; ++k) t += w_s[k];
-    wsum = t;
+  if (RULE != 0) {
+    t = warp_sum(t);
+    if (lane == 0) wsum[warp] = t;
+    __syncthreads();
+    t = 0.f;
+    for (int w = 0; w < AGG_THREADS / 32; ++w) t += wsum[w];
+    const float inv_w = 1.0f / t;
+    for (int k = tid; k < N; k += AGG_THREADS) wn_s[k] = w_s[k] * inv_w;
   }
   __syncthreads();
-  const float inv_w = 1.0f / wsum;
-  const float* lp0 = a.lp + (int64_t)b * n1 * V;
+  for (int k0 = 0; k0 < N; k0 += AGG_ROWS) {
+    float x[AGG_ROWS][AGG_TOK];
+#pragma unroll
+    for (int u = 0; u < AGG_ROWS; ++u)
+#pragma unroll
+      for (int j = 0; j < AGG_TOK; ++j) {
+        const int v = v0 + j * AGG_THREADS;
+        x[u][j] = k0 + u < N && v < V ? lp0[(int64_t)(k0 + u + 1) * V + v] : 0.f;
+      }
+#pragma unroll
+    for (int u = 0; u < AGG_ROWS; ++u) {
+      const int k = k0 + u;
+      if (k >= N) break;
+      const float bk = beta_s[k], lk = lse_s[k], wk = RULE == 0 ? 0.f : wn_s[k];
+#pragma unroll
+      for (int j = 0; j < AGG_TOK; ++j) {
+        const float ck = (1.f + bk) * x[u][j] - bk * l0[j];
+        if (RULE == 0)
+          acc[j] = fmaxf(acc[j], ck + lk);
+        else if (RULE == 1)
+          acc[j] += wk * expf(ck - lk);  // ck - lk = log p_k(v)
+        else
+          acc[j] += wk * (ck - lk);
+      }
+    }
+  }
   // the chunk's best aggregate and token, and the best at another token
   float bv = -INFINITY, b2 = -INFINITY;
   int bt = 0x7fffffff;
-  const int v1 = min(V, (c + 1) * AGG_CHUNK);
-  for (int v = c * AGG_CHUNK + tid; v < v1; v += AGG_THREADS) {
-    const float l0 = lp0[v];
-    float acc = a.rule == 0 ? -INFINITY : 0.f;
-    for (int k = 0; k < N; ++k) {
-      if (a.rule == 0) {
-        acc = fmaxf(acc, (1.f + beta_s[k]) * lp0[(int64_t)(k + 1) * V + v] - beta_s[k] * l0 + lse_s[k]);
-        continue;
-      }
-      const float lpk = (1.f + beta_s[k]) * lp0[(int64_t)(k + 1) * V + v] - beta_s[k] * l0 - lse_s[k];  // log p_k(v)
-      acc += a.rule == 1 ? w_s[k] * inv_w * expf(lpk) : w_s[k] * inv_w * lpk;
-    }
-    const float agg = a.rule == 1 ? logf(acc) : acc;
-    agg_top2(bv, bt, b2, agg, v, -INFINITY);
-  }
+#pragma unroll
+  for (int j = 0; j < AGG_TOK; ++j)
+    if (v0 + j * AGG_THREADS < V)
+      agg_top2(bv, bt, b2, RULE == 1 ? logf(acc[j]) : acc[j], v0 + j * AGG_THREADS, -INFINITY);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float v2 = __shfl_xor_sync(0xffffffffu, bv, o), s2 = __shfl_xor_sync(0xffffffffu, b2, o);
@@ -213,7 +270,7 @@ __global__ void __launch_bounds__(AGG_THREADS) agg_select_kernel(AggArgs a) {
   int bk = 0x7fffffff;
   for (int k = lane; k < N; k += 32) {
     const float ck = (1.f + beta_s[k]) * lp0[(int64_t)(k + 1) * V + st] - beta_s[k] * lp0[st];
-    agg_top2(bp, bk, bp2, a.rule == 0 ? ck + lse_s[k] : logf(w_s[k]) + ck - lse_s[k], k, -INFINITY);
+    agg_top2(bp, bk, bp2, RULE == 0 ? ck + lse_s[k] : logf(w_s[k]) + ck - lse_s[k], k, -INFINITY);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -222,10 +279,10 @@ __global__ void __launch_bounds__(AGG_THREADS) agg_select_kernel(AggArgs a) {
     agg_top2(bp, bk, bp2, v2, t2, s2);
   }
   if (bk >= N) bk = 0;
+  if (a.lse_out)
+    for (int j = lane; j < n1; j += 32) a.lse_out[b * n1 + j] = a.lse[b * n1 + j];
   if (lane != 0) return;
   a.qdone[b] = 0;
-  if (a.lse_out)
-    for (int j = 0; j < n1; ++j) a.lse_out[b * n1 + j] = a.lse[b * n1 + j];
   if (a.key_out) {  // expert-partitioned step (rule 0): the reduction and the append come after
     a.key_out[b] = select_key(sv, st, a.expert_base + bk + 1);
     return;
@@ -252,14 +309,14 @@ __global__ void __launch_bounds__(AGG_THREADS) agg_select_kernel(AggArgs a) {
   }
 }
 
-cudaError_t agg_partials_launch(const AggArgs& a, cudaStream_t stream) {
-  agg_partials_kernel<<<dim3(a.nchunks, a.N, a.B), AGG_THREADS, 0, stream>>>(a);
-  return cudaGetLastError();
+cudaError_t agg_partials_launch(const AggArgs& a, bool pdl, cudaStream_t stream) {
+  const int nc = pced_host::row_cluster((int64_t)a.B * a.N);
+  return pced_host::launch_cluster(agg_partials_kernel, dim3(nc, a.N, a.B), nc, AGG_L_THREADS, 0, stream, pdl, a);
 }
 
-cudaError_t agg_select_launch(const AggArgs& a, cudaStream_t stream) {
-  agg_select_kernel<<<dim3(a.nchunks, a.B), AGG_THREADS, 0, stream>>>(a);
-  return cudaGetLastError();
+cudaError_t agg_select_launch(const AggArgs& a, bool pdl, cudaStream_t stream) {
+  auto kernel = a.rule == 0 ? agg_select_kernel<0> : a.rule == 1 ? agg_select_kernel<1> : agg_select_kernel<2>;
+  return pced_host::launch_kernel(kernel, dim3(a.nchunks, a.B), AGG_THREADS, 0, stream, pdl, a);
 }
 
 }  // namespace pced

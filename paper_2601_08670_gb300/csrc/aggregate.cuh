@@ -20,8 +20,6 @@ struct AggArgs {
   int32_t B, N, V, rule, nchunks;  // rule 0 Eq. 3 (max over experts), 1 MoE, 2 PoE
   float gamma;          // rule 0: weight of the retrieval prior
   int raw_logits;       // rule 0: s_k of Eq. 2 are the raw logits lp + lse
-  float2* part;         // [B][N][nchunks] (max, sum exp) of c_k over each chunk
-  int32_t* kdone;       // [B][N] chunks finished per expert (zero at launch; the last resets it)
   float* lse_k;         // [B][N] log-sum-exp of c_k (the softmax normaliser of p_k)
   float2* best;         // [B][nchunks] (aggregate, token) of each chunk
   float* best2;         // [B][nchunks] the chunk's best aggregate at another token
@@ -47,8 +45,9 @@ struct AggArgs {
 constexpr int AGG_CHUNK = 1024;  // vocabulary entries per CTA (about 125 CTAs per query at V = 128K)
 constexpr int AGG_MAX_N = 512;   // experts per query (the LM head's row limit)
 inline int32_t agg_chunks(int32_t V) { return (V + AGG_CHUNK - 1) / AGG_CHUNK; }
-// (1) per (query, expert, chunk) statistics, (2) per (query, chunk) best and the pick
-cudaError_t agg_partials_launch(const AggArgs& a, cudaStream_t stream);
-cudaError_t agg_select_launch(const AggArgs& a, cudaStream_t stream);
+// (1) per (query, expert) log-sum-exp, (2) per (query, chunk) best and the pick
+// (pdl: as programmatic dependents)
+cudaError_t agg_partials_launch(const AggArgs& a, bool pdl, cudaStream_t stream);
+cudaError_t agg_select_launch(const AggArgs& a, bool pdl, cudaStream_t stream);
 
 }  // namespace pced

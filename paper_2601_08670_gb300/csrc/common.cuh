@@ -508,6 +508,8 @@ __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2
   m = M;
 }
 
+constexpr int ROW_CLUSTER = 8;  // most CTAs of a cluster that shares a row of the vocabulary
+
 }  // namespace pced
 
 // ------------------------------------------------------------------- host side
@@ -527,6 +529,14 @@ pced_status make_tmap_kv(CUtensorMap* map, const void* base, uint64_t rows, uint
 // kernel.  Every kernel launched so calls pdl_wait() in all of its threads
 // before it touches memory that an earlier launch may write or still read, so
 // only its launch, and what it does before the wait, overlap that kernel.
+// CTAs per (query, expert) of the kernels that read an expert's and the
+// amateur's row of the vocabulary: a cluster of up to ROW_CLUSTER, fewer from
+// two CTAs per SM on, where a longer part of the row per CTA pays for its
+// reduction (16 x 16 rows of 128256 entries: log-sum-exp 59 us with one CTA a
+// row, 68 with two, 79 with eight; 64 rows: beta 24 us with four, 27 with eight,
+// 41 with two).
+int row_cluster(int64_t rows);
+
 template <typename... P>
 cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int cluster, unsigned threads, size_t smem,
                            cudaStream_t stream, bool pdl, P... args) {

@@ -50,6 +50,12 @@ int num_sms() {
   return cache[dev];
 }
 
+int row_cluster(int64_t rows) {
+  int nc = pced::ROW_CLUSTER;
+  while (nc > 1 && rows * nc > 2 * (int64_t)num_sms()) nc >>= 1;
+  return nc;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -29,10 +29,8 @@ struct StepLayout {
   int32_t* lm_tile_ctr;   // LM head: vocabulary tiles claimed (reset by the selection)
   float* sel_L;           // log-sum-exps of the rows (dynamic beta, MoE / PoE)
   float* lp;              // [S][V] log-probabilities of a dynamic-beta first step
-  float2* agg_part;       // MoE / PoE: per (query, expert, chunk) statistics
   float2* agg_best;       // MoE / PoE: per (query, chunk) best
   float* agg_best2;       // MoE / PoE: per (query, chunk) best at another token
-  int32_t* agg_kdone;     // MoE / PoE: chunks finished per (query, expert)
   float* agg_lse;         // MoE / PoE: per (query, expert) log-sum-exp of the contrastive scores
   int32_t* agg_qdone;     // MoE / PoE: chunks finished per query
   uint64_t* part_ss;
@@ -69,10 +67,8 @@ static StepLayout step_layout(const pced_dims* dm, void* ws) {
   L.lm_tile_ctr = c.take<int32_t>(1);
   L.sel_L = c.take<float>((size_t)S);
   L.lp = c.take<float>((size_t)S * dm->V);
-  L.agg_part = c.take<float2>((size_t)dm->B * dm->N * agg_chunks(dm->V));
   L.agg_best = c.take<float2>((size_t)dm->B * agg_chunks(dm->V));
   L.agg_best2 = c.take<float>((size_t)dm->B * agg_chunks(dm->V));
-  L.agg_kdone = c.take<int32_t>((size_t)dm->B * dm->N);
   L.agg_lse = c.take<float>((size_t)dm->B * dm->N);
   L.agg_qdone = c.take<int32_t>((size_t)dm->B);
   L.bytes = c.used() + 4 * (4096 - 256);  // room for the 4 KB alignment of four arrays
@@ -348,10 +344,8 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     ag.gamma = p->gamma;
     ag.raw_logits = p->score_mode == PCED_SCORE_LOGIT;
     ag.nchunks = agg_chunks(dm.V);
-    ag.part = W.agg_part;
     ag.best = W.agg_best;
     ag.best2 = W.agg_best2;
-    ag.kdone = W.agg_kdone;
     ag.lse_k = W.agg_lse;
     ag.gap_trace = p->key_out ? nullptr : reinterpret_cast<float2*>(p->gap_trace);
     ag.key_out = p->key_out;
@@ -371,11 +365,11 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     ag.status = W.status;
     if (agg) {
       ranges.next("agg_partials");
-      e = agg_partials_launch(ag, s);
+      e = agg_partials_launch(ag, !timed, s);
       if (e == cudaSuccess) e = mark();
     }
     if (e == cudaSuccess) ranges.next("agg_select");
-    if (e == cudaSuccess) e = agg_select_launch(ag, s);
+    if (e == cudaSuccess) e = agg_select_launch(ag, !timed, s);
     if (e == cudaSuccess) e = mark();
     if (e != cudaSuccess) return cuda_status(e, "aggregation launches");
     return PCED_OK;
