@@ -127,8 +127,14 @@ def _ptr(t):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    """The raw handle of `stream`, by default of the current stream (asked for
+    directly: building the torch.cuda.Stream object costs 3 us per call, a
+    quarter of what a small call takes on the host)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def workspace(nbytes: int, device) -> torch.Tensor:
