@@ -1573,8 +1573,8 @@ size_t att_records_bytes(int32_t S, int32_t Hq, int32_t Hkv, int32_t D) {
   return c.used();
 }
 
-int att_grid(int64_t total_cap_keys) {
-  int64_t want = (total_cap_keys + 255) / 256;
+int att_grid(int64_t total_cap_keys, int keys_per_cta) {
+  int64_t want = (total_cap_keys + keys_per_cta - 1) / keys_per_cta;
   int64_t sms = pced_host::num_sms();
   int64_t g = want < sms ? want : sms;
   if (g > ATT_MAX_CTAS) g = ATT_MAX_CTAS;
@@ -1591,7 +1591,16 @@ static int env_int(const char* name, int dflt, int lo, int hi) {
 }
 int att_step_seg_cost(int D) { return env_int("PCED_ATT_SEGCOST", 512, 0, 1 << 20); }
 int att_step_pf_tiles() { return env_int("PCED_ATT_PF", 6, 0, 64); }
-int att_step_groups() { return env_int("PCED_ATT_GROUPS", 2, 1, ATT_MAX_GROUPS); }
+// Two groups, the second of which streams while the first one's layer dependency
+// resolves (eight layers of 9 sequences of 2080 rows: 120 us against 137 with
+// one); one group where there are many more segments than CTAs, so that few
+// are split, CTAs hardly wait for one another and the second group's pieces
+// only cost (two layers of 272 sequences around 1184 rows: 449 us against 469,
+// of 65 sequences of 544 rows 77 against 82; equal within 1 % at 1.7 segments
+// per CTA).
+int att_step_groups(int32_t S, int32_t Hkv, int ctas) {
+  return env_int("PCED_ATT_GROUPS", (int64_t)S * Hkv > 3 * (int64_t)ctas ? 1 : 2, 1, ATT_MAX_GROUPS);
+}
 int att_step_seg_lead(int seg_cost) { return env_int("PCED_ATT_LEAD", seg_cost / 2, 0, seg_cost); }
 
 // cudaFuncSetAttribute once per kernel and device
@@ -1621,7 +1630,7 @@ static cudaError_t launch_split(const CUtensorMap& kmap, const CUtensorMap& vmap
 
 cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, AttArgs a, int64_t total_cap_keys,
                              void* scratch, cudaStream_t stream) {
-  int ctas = att_grid(total_cap_keys);
+  int ctas = att_grid(total_cap_keys, 128);
   if (ctas > ATT_SPLIT_CTAS) ctas = ATT_SPLIT_CTAS;
   pced_host::Carver cv(scratch);
   a.rec_o = cv.take<float>((size_t)2 * ctas * a.G * D);

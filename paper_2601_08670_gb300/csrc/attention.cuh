@@ -53,7 +53,7 @@ struct CombineArgs {
 
 constexpr int ATT_SPLIT_CTAS = ATT_MAX_CTAS / 4;  // grid limit (2 records per CTA fit what att_records_bytes gives)
 size_t att_records_bytes(int32_t S, int32_t Hq, int32_t Hkv, int32_t D);
-int att_grid(int64_t total_cap_keys);
+int att_grid(int64_t total_cap_keys, int keys_per_cta);  // a CTA for so many keys, up to one per SM
 // one layer's split and combine kernels, for head dim D (64 or 128); records and
 // plan (rec_o, rec_ml, plan of `a`) are placed in `scratch`, 256-byte aligned
 cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, AttArgs a, int64_t total_cap_keys,
@@ -135,7 +135,7 @@ int64_t att_step_slots(int32_t S, int32_t Hkv);
 // PCED_ATT_PF in the environment override the defaults)
 int att_step_seg_cost(int D);
 int att_step_pf_tiles();
-int att_step_groups();
+int att_step_groups(int32_t S, int32_t Hkv, int ctas);
 int att_step_seg_lead(int seg_cost);
 cudaError_t att_step_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, const StepAttArgs& a, int ctas,
                             cudaStream_t stream);

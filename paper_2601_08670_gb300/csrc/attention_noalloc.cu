@@ -86,11 +86,13 @@ extern "C" pced_status pced_decode_attention_noalloc(const void* q, const void* 
     return fail(PCED_ERR_INVALID_ARG, "pced_decode_attention_noalloc: status must be 4-byte aligned");
   if (num_sms() <= 0) return fail(PCED_ERR_NO_DEVICE, "pced_decode_attention_noalloc: no CUDA device");
 
-  // The documented limit on sizes: (CTAs + S*Hkv) records and a prefix table.
-  // What a call uses of the array is less: the status sink, then the 2
-  // records per CTA and the plan that att_layer_launch places.
+  // The documented limit on sizes: a record for every segment and CTA (one CTA
+  // for every 256 keys, up to one per SM) and a prefix table.  What a call
+  // uses of the array is less: the status sink, then the 2 records per CTA
+  // and the plan that att_layer_launch places.
   const int32_t G = Hq / Hkv;
-  const int ctas = att_grid(total_cap * Hkv);
+  const int64_t want = (total_cap * Hkv + 255) / 256, sms = num_sms();
+  const int ctas = (int)(want < sms ? want : sms);
   const int64_t slots = (int64_t)ctas + (int64_t)S * Hkv;
   Carver sizer(nullptr);
   sizer.take<int32_t>(1);
