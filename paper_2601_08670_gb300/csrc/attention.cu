@@ -623,32 +623,41 @@ struct GroupPlan {
 // power of two dividing every extent): CTA c of a group takes positions
 // [c*P, (c+1)*P) rounded down to multiples of align, with P at least align,
 // so every CTA range is a whole number of tiles and none inside a segment is
-// empty (the CTAs holding a segment's keys stay consecutive).
+// empty (the CTAs holding a segment's keys stay consecutive).  One warp.
 __device__ __forceinline__ void plan_groups(GroupPlan& gp, const int64_t* pre, int32_t S, int32_t Hkv, int want,
-                                            int64_t grid, int64_t cta, int32_t align = 1) {
+                                            int64_t grid, int64_t cta, int lane, int32_t align = 1) {
   int ng = want < 1 ? 1 : (want > ATT_MAX_GROUPS ? ATT_MAX_GROUPS : want);
   if (ng > S) ng = S;
   const int64_t T = pre[S];
-  gp.s_lo[0] = 0;
-  for (int g = 1; g < ng; ++g) {
-    const int64_t target = T * g / ng;
-    int32_t s = gp.s_lo[g - 1] + 1;
-    while (s < S - (ng - g) && pre[s] < target) ++s;
-    gp.s_lo[g] = s;
+  if (lane == 0) {
+    gp.n = ng;
+    gp.s_lo[0] = 0;
+    for (int g = 1; g < ng; ++g) {
+      // the first sequence that starts at or past the target, after the
+      // previous group's first and leaving one for each group to come
+      const int64_t target = udiv_pos(T * g, ng);
+      int32_t lo = gp.s_lo[g - 1] + 1, hi = S - (ng - g);
+      while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (pre[mid] < target) lo = mid + 1;
+        else hi = mid;
+      }
+      gp.s_lo[g] = lo;
+    }
+    gp.s_lo[ng] = S;
   }
-  gp.s_lo[ng] = S;
-  for (int g = 0; g < ng; ++g) {
-    const int64_t Tg = pre[gp.s_lo[g + 1]] - pre[gp.s_lo[g]];
+  __syncwarp();
+  if (lane < ng) {
+    const int64_t Tg = pre[gp.s_lo[lane + 1]] - pre[gp.s_lo[lane]];
     const int64_t tot = (int64_t)Hkv * Tg;
-    int64_t Pg = (tot + grid - 1) / grid;
+    int64_t Pg = udiv_pos(tot + grid - 1, grid);
     if (Pg < align) Pg = align;
     const int64_t am = ~(int64_t)(align - 1);
-    gp.T[g] = Tg;
-    gp.P[g] = Pg;
-    gp.cb[g] = min(tot, cta * Pg) & am;
-    gp.ce[g] = min(tot, (cta + 1) * Pg) & am;
+    gp.T[lane] = Tg;
+    gp.P[lane] = Pg;
+    gp.cb[lane] = min(tot, cta * Pg) & am;
+    gp.ce[lane] = min(tot, (cta + 1) * Pg) & am;
   }
-  gp.n = ng;
 }
 
 // Block index of key x (paged caches).
@@ -893,12 +902,11 @@ struct PieceDesc {
 // aligned base), a function of the head dim and group size only.
 struct StepSmem {
   uint32_t stages;      // K/V ring stages
-  uint32_t bar;         // full[st] empty[st] qfull[2] qempty[2] pfull[2] pempty[2] msync
+  uint32_t bar;         // full[st] empty[st] qfull[2] qempty[2] pfull[2] pempty[2]
   uint32_t qbuf, qslot; // [2] hand-off slots: q words [8][D/2+4], K row, V row (bf16), x_l of the head group (fp32),
                         // PieceDesc (at qdesc)
   uint32_t qdesc;
   uint32_t pbuf, pslot; // [2] partial hand-off slots: ms[8][8], ls[8][8], os[8][G][D + 4]
-  uint32_t misc;        // flags
   uint32_t tables;      // pre[ATT_MAX_S+1] int64, GroupPlan, lens[ATT_MAX_S] int32, apnd[ATT_MAX_S] u8
   uint32_t ptab;        // block-table copy: ptab[ATT_PTAB] int32, its entry count, ptab_h[ATT_PTAB] u8
   uint32_t rope;        // rotary inverse frequencies [D/2] fp32
@@ -917,8 +925,7 @@ __host__ __device__ inline StepSmem step_smem(int D, int G) {
     L.qbuf = L.bar + (2u * L.stages + 9u) * 8u;
     L.qbuf = (L.qbuf + 15u) & ~15u;
     L.pbuf = L.qbuf + 2u * L.qslot;
-    L.misc = L.pbuf + 2u * L.pslot;
-    L.tables = L.misc + 64u;
+    L.tables = L.pbuf + 2u * L.pslot + 64u;
     L.ptab = L.tables + ((tables + 15u) & ~15u);
     L.rope = (L.ptab + ATT_PTAB * 5u + 16u + 15u) & ~15u;
     L.total = 1024u + L.rope + 4u * (uint32_t)(D / 2);
@@ -995,8 +1002,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
   const uint32_t NST = SL.stages;
   const uint32_t bar_full = base + SL.bar, bar_empty = bar_full + 8 * NST;
   const uint32_t bar_qfull = bar_empty + 8 * NST, bar_qempty = bar_qfull + 16;
-  const uint32_t bar_pfull = bar_qempty + 16, bar_pempty = bar_pfull + 16, bar_m = bar_pempty + 16;
-  int* flag = reinterpret_cast<int*>(gbase + SL.misc + 32);
+  const uint32_t bar_pfull = bar_qempty + 16, bar_pempty = bar_pfull + 16;
   int64_t* pre = reinterpret_cast<int64_t*>(gbase + SL.tables);
   GroupPlan& gp = *reinterpret_cast<GroupPlan*>(pre + ATT_MAX_S + 1);
   int32_t* lens = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(&gp) + ((sizeof(GroupPlan) + 7) & ~(size_t)7));
@@ -1020,7 +1026,6 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
       mbar_init(bar_pfull + 8 * i, ATT_CONSUMERS);
       mbar_init(bar_pempty + 8 * i, ATT_CONSUMERS);
     }
-    mbar_init(bar_m, ATT_CONSUMERS);
     mbar_fence_init();
   }
   if (warp == STEP_PRODUCER && lane == 0) {
@@ -1030,31 +1035,41 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
   // the next grid (LM head) may be scheduled as SMs free up; it waits for
   // this grid's completion before reading the hidden states
   pdl_launch_dependents();
-  // rotary inverse frequencies theta^(-2f/D), rounded to fp32
-  if (a.rope_theta > 0.f && tid < D / 2) rope_f[tid] = (float)pow((double)a.rope_theta, -2.0 * tid / D);
-  // lengths after this step's append (a full cache appends nothing)
-  for (int i = tid; i < S; i += STEP_THREADS) {
-    int32_t n = a.seq_len[i];
-    const int32_t c = a.cap[i];
-    if (n < 0 || n > c) {
-      dev_flag(a.status, PCED_DEV_BAD_LENGTH);
-      n = n < 0 ? 0 : c;
-    }
-    const bool ap = n < c;
-    if (!ap) dev_flag(a.status, PCED_DEV_CACHE_FULL);
-    int32_t len = ap ? n + 1 : n;
-    if (len < 1) {
-      dev_flag(a.status, PCED_DEV_BAD_LENGTH);
-      len = 1;
-    }
-    lens[i] = len;
-    apnd[i] = ap ? 1 : 0;
-  }
-  __syncthreads();
   const int32_t align = a.block_table ? ATT_BLOCK_N : 1;
-  if (warp == 0) prefix_extents(lens, S, a.seg_cost, pre, lane, align);
-  __syncthreads();
-  if (tid == 0) plan_groups(gp, pre, S, Hkv, a.groups, gridDim.x, blockIdx.x, align);
+  if (warp == STEP_INPUT) {
+    // x_0 needs neither the lengths nor the partition: its loads go out before
+    // the first tiles fill the memory system (embedded after the partition,
+    // the first query was ready 13.7 us after the start of a 4-layer launch
+    // and 8.3 us after that of the tiny one)
+    embed_slices<D>(a, step_tag(epoch, 0), lane);
+  } else {
+    // rotary inverse frequencies theta^(-2f/D), rounded to fp32
+    if (a.rope_theta > 0.f && tid < D / 2) rope_f[tid] = (float)pow((double)a.rope_theta, -2.0 * tid / D);
+    // lengths after this step's append (a full cache appends nothing)
+    for (int i = tid; i < S; i += STEP_THREADS - 32) {
+      int32_t n = a.seq_len[i];
+      const int32_t c = a.cap[i];
+      if (n < 0 || n > c) {
+        dev_flag(a.status, PCED_DEV_BAD_LENGTH);
+        n = n < 0 ? 0 : c;
+      }
+      const bool ap = n < c;
+      if (!ap) dev_flag(a.status, PCED_DEV_CACHE_FULL);
+      int32_t len = ap ? n + 1 : n;
+      if (len < 1) {
+        dev_flag(a.status, PCED_DEV_BAD_LENGTH);
+        len = 1;
+      }
+      lens[i] = len;
+      apnd[i] = ap ? 1 : 0;
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(STEP_THREADS - 32) : "memory");  // all warps but the input warp
+    if (warp == 0) {
+      prefix_extents(lens, S, a.seg_cost, pre, lane, align);
+      __syncwarp();
+      plan_groups(gp, pre, S, Hkv, a.groups, gridDim.x, blockIdx.x, lane, align);
+    }
+  }
   __syncthreads();
   if (a.block_table) {
     // paged caches: for the blocks of this CTA's pieces (the same in every
@@ -1108,7 +1123,6 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
     // group sums of x_l[s], then hand the consumers q = bf16(x_l * inv_rms)
     // (and, for the piece holding the row appended this step, that row's K
     // and V, also written to the caches) through a double-buffered slot.
-    embed_slices<D>(a, step_tag(epoch, 0), lane);
     uint32_t p = 0;
     bool ok = true;
     for (int l = 0; l < a.L && ok; ++l) {
@@ -1154,6 +1168,12 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         static_assert(32 % (D / 4) == 0, "rotary quads per lane assume D/4 divides 32");
         RopePair rp = {1.f, 0.f, 1.f, 0.f};
         if (rope) rp = rope_angles(2 * (lane % (D / 4)), (float)(lens[pc.s] - apnd[pc.s]), rope_f);
+        // K row = head h of u (rotated like the queries), V row = head Hkv + h of
+        // u: a rotary quad per lane, loaded with the first chunk
+        const uint64_t* xk = xs + (int64_t)pc.h * D;
+        const uint64_t* xv = xs + ((int64_t)Hkv + pc.h) * D;
+        const bool kv = app && lane < D / 4;
+        float kx[4] = {0.f, 0.f, 0.f, 0.f}, vx[4] = {0.f, 0.f, 0.f, 0.f};
         for (int m0 = 0; m0 < GD / 4 && ok; m0 += 32 * 4) {
           float v[4][4], t = 0.f;
           uint64_t t0 = 0;
@@ -1166,6 +1186,16 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
                 good &= tv_ok(w, tag);
                 t += tv_value(w);
               }
+            if (m0 == 0 && kv) {
+              const int e[4] = {2 * lane, 2 * lane + 1, 2 * lane + D / 2, 2 * lane + 1 + D / 2};
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const uint64_t wk = ld_tagged(xk + e[c]), wv = ld_tagged(xv + e[c]);
+                good &= tv_ok(wk, tag) && tv_ok(wv, tag);
+                kx[c] = tv_value(wk);
+                vx[c] = tv_value(wv);
+              }
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const int m = m0 + lane + 32 * j;
@@ -1208,75 +1238,20 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
             xr[e + D / 2 + 1] = v[j][3];
           }
         }
-        if (ok && app) {
-          // K row = head h of u (rotated like the queries), V row = head Hkv + h of u
-          const uint64_t* xk = xs + (int64_t)pc.h * D;
-          const uint64_t* xv = xs + ((int64_t)Hkv + pc.h) * D;
+        uint32_t ka = 0, kc = 0, va = 0, vc = 0;  // this lane's words of the appended rows
+        if (ok && kv) {
+          float a0 = kx[0] * inv, a1 = kx[1] * inv, b0 = kx[2] * inv, b1 = kx[3] * inv;
+          if (rope) rope_rotate(a0, a1, b0, b1, rp);  // keys rotate, values do not
+          ka = pack_bf16(a0, a1);
+          kc = pack_bf16(b0, b1);
+          va = pack_bf16(vx[0] * inv, vx[1] * inv);
+          vc = pack_bf16(vx[2] * inv, vx[3] * inv);
           uint32_t* kr = qw + 8 * QW;
           uint32_t* vr = kr + D / 2;
-          int64_t arow;
-          if (a.block_table) {
-            const int32_t key = lens[pc.s] - 1, j = block_of(a, key);
-            const int32_t b0 = block_base(a, pc.s, pc.h, j, pt + (j - j0), ptab, ptab_n);
-            arow = b0 < 0 ? -1 : (int64_t)l * a.rows_per_layer + b0 + (key - j * a.block_rows);
-          } else {
-            arow = (int64_t)l * a.rows_per_layer + (a.kv_offset[pc.s] + (int64_t)pc.h * a.cap[pc.s] * D) / D +
-                   lens[pc.s] - 1;
-          }
-          // a bad block id was flagged: keep the cache untouched
-          const bool wrow = arow >= 0 &&
-                            PCED_IN_BOUNDS(arow >= (int64_t)l * a.rows_per_layer &&
-                                               arow < (int64_t)(l + 1) * a.rows_per_layer &&
-                                               (a.block_table || lens[pc.s] - 1 < a.cap[pc.s]),
-                                           a.status);
-          const int64_t grow = (wrow ? arow : 0) * D;
-          constexpr int RQ = (D / 4 + 31) / 32;  // rotary quads per lane (as for the queries)
-          float kx[RQ][4], vx[RQ][4];
-          uint64_t t0 = 0;
-          while (true) {
-            bool good = true;
-#pragma unroll
-            for (int j = 0; j < RQ; ++j) {
-              const int k = lane + 32 * j;
-#pragma unroll
-              for (int c = 0; c < 4; ++c) kx[j][c] = vx[j][c] = 0.f;
-              if (k >= D / 4) continue;
-              const int e[4] = {2 * k, 2 * k + 1, 2 * k + D / 2, 2 * k + 1 + D / 2};
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const uint64_t wk = ld_tagged(xk + e[c]), wv = ld_tagged(xv + e[c]);
-                good &= tv_ok(wk, tag) && tv_ok(wv, tag);
-                kx[j][c] = tv_value(wk);
-                vx[j][c] = tv_value(wv);
-              }
-            }
-            if (__all_sync(0xffffffffu, good)) break;
-            if (!poll_again(t0, a.status, a.wait_ns)) {
-              ok = false;
-              break;
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < RQ; ++j) {
-            const int k = lane + 32 * j;
-            if (!ok || k >= D / 4) continue;
-            float a0 = kx[j][0] * inv, a1 = kx[j][1] * inv, b0 = kx[j][2] * inv, b1 = kx[j][3] * inv;
-            if (rope) rope_rotate(a0, a1, b0, b1, rp);  // keys rotate, values do not
-            const uint32_t ka = pack_bf16(a0, a1), kb = pack_bf16(b0, b1);
-            const uint32_t va = pack_bf16(vx[j][0] * inv, vx[j][1] * inv), vb = pack_bf16(vx[j][2] * inv, vx[j][3] * inv);
-            kr[k] = ka;
-            kr[k + D / 4] = kb;
-            vr[k] = va;
-            vr[k + D / 4] = vb;
-            if (wrow) {
-              uint32_t* gk = reinterpret_cast<uint32_t*>(a.k_cache + grow);
-              uint32_t* gv = reinterpret_cast<uint32_t*>(a.v_cache + grow);
-              gk[k] = ka;
-              gk[k + D / 4] = kb;
-              gv[k] = va;
-              gv[k + D / 4] = vb;
-            }
-          }
+          kr[lane] = ka;
+          kr[lane + D / 4] = kc;
+          vr[lane] = va;
+          vr[lane + D / 4] = vc;
         }
         if (lane == 0) {
           const int64_t pa = (int64_t)pc.h * gp.T[gi] + pre[pc.s] - pre[gp.s_lo[gi]] + a.seg_lead;  // first key
@@ -1294,6 +1269,33 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_qfull + 8 * slot);
+        if (ok && app) {
+          // the appended rows into the caches (the consumers have theirs from
+          // the slot, so the address is found after the hand-off)
+          int64_t arow;
+          if (a.block_table) {
+            const int32_t key = lens[pc.s] - 1, j = block_of(a, key);
+            const int32_t b0 = block_base(a, pc.s, pc.h, j, pt + (j - j0), ptab, ptab_n);
+            arow = b0 < 0 ? -1 : (int64_t)l * a.rows_per_layer + b0 + (key - j * a.block_rows);
+          } else {
+            arow = (int64_t)l * a.rows_per_layer + (a.kv_offset[pc.s] + (int64_t)pc.h * a.cap[pc.s] * D) / D +
+                   lens[pc.s] - 1;
+          }
+          // a bad block id was flagged: keep the cache untouched
+          const bool wrow = arow >= 0 &&
+                            PCED_IN_BOUNDS(arow >= (int64_t)l * a.rows_per_layer &&
+                                               arow < (int64_t)(l + 1) * a.rows_per_layer &&
+                                               (a.block_table || lens[pc.s] - 1 < a.cap[pc.s]),
+                                           a.status);
+          if (wrow && kv) {
+            uint32_t* gk = reinterpret_cast<uint32_t*>(a.k_cache + arow * D);
+            uint32_t* gv = reinterpret_cast<uint32_t*>(a.v_cache + arow * D);
+            gk[lane] = ka;
+            gk[lane + D / 4] = kc;
+            gv[lane] = va;
+            gv[lane + D / 4] = vc;
+          }
+        }
       }
       }
     }
@@ -1312,6 +1314,20 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
   }
 
   // -------------------------------------------------------------- consumers
+  // Every CTA has read the lengths and the epoch; the last one to say so
+  // advances them, while its consumers wait for the first query (at the end of
+  // the launch the round trip of this counter cost 1.1 us)
+  if (warp == ATT_CONSUMERS - 1) {
+    const int prev = lane == 0 ? atom_acq_rel_gpu_add(a.done_cnt, 1) : 0;
+    if (__shfl_sync(0xffffffffu, prev, 0) == (int)gridDim.x - 1) {
+      for (int i = lane; i < S; i += 32)
+        if (apnd[i]) a.seq_len[i] = lens[i];
+      if (lane == 0) {
+        *a.done_cnt = 0;
+        *a.epoch = epoch + 1;
+      }
+    }
+  }
   const int wg = warp >> 2, wl = warp & 3;
   const int g = lane >> 2, tq = lane & 3;
   const int kb = 16 * wl;
@@ -1541,20 +1557,6 @@ __global__ void __launch_bounds__(STEP_THREADS, 1)
           }
         }
       }
-    }
-  }
-  // ---- the last CTA to finish advances seq_len and the epoch
-  uint32_t cph = 0;
-  if (tid == 0) {
-    const int prev = atom_acq_rel_gpu_add(a.done_cnt, 1);
-    flag[0] = prev == (int)gridDim.x - 1;
-  }
-  if (warps_sync(bar_m, cph, a.status) && flag[0]) {
-    for (int i = tid; i < S; i += ATT_CT)
-      if (apnd[i]) a.seq_len[i] = lens[i];
-    if (tid == 0) {
-      *a.done_cnt = 0;
-      *a.epoch = epoch + 1;
     }
   }
 }
