@@ -29,6 +29,9 @@ struct LmGeom {
 // returns false when the shape is unsupported
 bool lm_geometry(int32_t S, int32_t d, int32_t V, LmGeom* g);
 
+constexpr int LM_PDL_H = 1;    // of the kernel that writes H: the weights are read before it ends
+constexpr int LM_PDL_ALL = 2;  // of any kernel: nothing is read before it ends
+
 struct LmArgs {
   int mode;  // 0: write logits[S][V]; 1: contrastive records (needs N, beta)
   int32_t S, N, V, ntiles, nks, slabs, nst, stages, acc_bufs, S_pad;
@@ -39,9 +42,9 @@ struct LmArgs {
   float2* rec_stats;  // [S][ntiles] (max z, sum exp(z - max)) of each vocabulary tile
   float2* rec_arg;    // [S][ntiles] (max u, argmax v as int bits) for expert columns, mode 1
   float* rec_u2;      // [S][ntiles] the tile's second-largest u (another token), mode 1
-  int* tile_ctr;      // tiles claimed so far (zero at launch)
+  int* tile_ctr;      // tiles claimed so far (zero at launch), or null: dealt out in turn
   const float* beta;  // [B][N]
-  int pdl;            // launched as a programmatic dependent of the kernel that writes H
+  int pdl;            // launched as a programmatic dependent: LM_PDL_H, LM_PDL_ALL (0: not)
   int* status;
 };
 

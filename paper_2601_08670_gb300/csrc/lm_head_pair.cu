@@ -107,15 +107,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
     int tile = -1, ks = 0;
     uint32_t tseq = 0;
     bool ok = true;
-    // tile tseq of the pair: claimed by CTA 0 from the global counter and
-    // handed to both CTAs (-1 ends); a ring entry is used again LM_TRING
+    // tile tseq of the pair: claimed by CTA 0 from the global counter (without
+    // one, the pairs' tiles in turn) and handed to both CTAs (-1 ends); a ring entry is used again LM_TRING
     // tiles later, when every role of both CTAs is past it
     auto claim = [&]() {
       const uint32_t i = tseq % LM_TRING;
       int t = -1;
       if (rank == 0) {
         if (lane == 0) {
-          t = atomicAdd(a.tile_ctr, 1);
+          t = a.tile_ctr ? atomicAdd(a.tile_ctr, 1) : (int)((blockIdx.x >> 1) + tseq * (gridDim.x >> 1));
           if (t >= ntiles) t = -1;
           tring[i] = t;
           st_cluster_u32(mapa(smem_u32(tring + i), 1), (uint32_t)t);
@@ -147,12 +147,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
                          n0 + (int)rank * (nc1 / 2), pol_h);
       if (++hks == nks) hks = 0;
     };
+    if (a.pdl == LM_PDL_ALL) pdl_wait();
     claim();
     // first fill; with programmatic dependent launch W streams while the
     // previous kernel (which writes H) finishes
     uint32_t nw = 0, nh = 0;  // slabs of W and of H issued
     while (tile >= 0 && nw < wst_n) load_w(nw++);
-    if (a.pdl) pdl_wait();
+    if (a.pdl == LM_PDL_H) pdl_wait();
     for (; nh < hst_n && nh < nw; ++nh) load_h(nh, nh);
     // with slab n consumed, its W stage takes slab n + wst_n and its H stage slab n + hst_n
     uint32_t w = 0, wph = 0, h = 0, hw = nh == wst_n ? 0 : nh;

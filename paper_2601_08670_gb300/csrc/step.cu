@@ -304,7 +304,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     lz.rec_stats = W.lm_stats;
     lz.tile_ctr = W.lm_tile_ctr;
     lz.status = W.status;
-    lz.pdl = timed ? 0 : 1;  // streams weights while the attention kernel finishes
+    lz.pdl = timed ? 0 : LM_PDL_H;  // streams weights while the attention kernel finishes
     ranges.next("lm_head");
     e = lm_head_launch(maps, g, lz, s);
     if (e == cudaSuccess) e = mark();
@@ -385,7 +385,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   la.tile_ctr = W.lm_tile_ctr;
   la.beta = beta;
   la.status = W.status;
-  la.pdl = (timed || dyn) ? 0 : 1;  // stage events between the launches would break the overlap
+  la.pdl = (timed || dyn) ? 0 : LM_PDL_H;  // stage events between the launches would break the overlap
   ranges.next("lm_head");
   e = lm_head_launch(maps, g, la, s);
   if (e == cudaSuccess) e = mark();
