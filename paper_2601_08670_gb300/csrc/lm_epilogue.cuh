@@ -114,11 +114,12 @@ __device__ __forceinline__ void bfly_top2(const float (&u)[NB], int tok, int lan
 // broadcast buffer; z_am carries the row's amateur logit from its query's
 // first column to the expert columns; ccoef / cmask hold each column's
 // (1 + beta, beta) and the amateur / expert column bits of each 32-column
-// block (the same for every tile).
-template <int NB>
+// block (the same for every tile).  `loaded` runs once the accumulator's
+// columns are in registers.
+template <int NB, class F>
 __device__ __forceinline__ void epi_block(const LmArgs& a, uint32_t taddr, int c0, int v, bool valid, int lane,
                                           int q, float* bc, float2* wst, float2* wag, float* wu2, const float2* ccoef,
-                                          const uint32_t* cmask, float& z_am) {
+                                          const uint32_t* cmask, float& z_am, F loaded) {
   const int S = a.S, S_pad = a.S_pad;
   float z[NB], t[NB];
   if (NB == 32)
@@ -127,6 +128,7 @@ __device__ __forceinline__ void epi_block(const LmArgs& a, uint32_t taddr, int c
     tmem_ld16(taddr, z);
   else
     tmem_ld8(taddr, z);
+  loaded();
   if (a.mode == 0 && valid) {
 #pragma unroll
     for (int i = 0; i < NB; ++i)

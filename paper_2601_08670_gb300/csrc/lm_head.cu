@@ -31,7 +31,7 @@ namespace pced {
 
 namespace cg = cooperative_groups;
 
-constexpr int LM_PAIR_HSTAGES = 4;  // most stages of a pair's H ring
+constexpr int LM_PAIR_HSTAGES = 5;  // most stages of a pair's H ring
 
 bool lm_geometry(int32_t S, int32_t d, int32_t V, LmGeom* g) {
   if (S < 1 || S > LM_MAX_S || d < LM_TILE_K || d % LM_TILE_K != 0 || V < 1) return false;
@@ -361,17 +361,25 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
       if (a.mode == 1 && kb0 < kb1 && (W * kb0) % n1 != 0)
         z_am = tmem_ld1(trow + W * kb0 - (W * kb0) % n1);  // the row's amateur logit of the open query
       float* wbc = bc + 64 * (warp - 2);
+      // the accumulator is free for the next tile's MMAs once this warp's last
+      // columns are in its registers
+      auto release = [&]() {
+        tc_fence_before();
+        mbar_arrive(bar_tempty + 8 * buf);
+      };
+      if (kb0 >= kb1) release();
       for (int kb = kb0; kb < kb1; ++kb) {
         const int c0 = W * kb;
+        auto loaded = [&]() {
+          if (kb + 1 == kb1) release();
+        };
         if (W == 8)
-          epi_block<8>(a, trow + c0, c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am);
+          epi_block<8>(a, trow + c0, c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am, loaded);
         else if (c0 + 32 <= S_pad && W == 32)
-          epi_block<32>(a, trow + c0, c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am);
+          epi_block<32>(a, trow + c0, c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am, loaded);
         else
-          epi_block<16>(a, trow + c0, c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am);
+          epi_block<16>(a, trow + c0, c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am, loaded);
       }
-      tc_fence_before();
-      mbar_arrive(bar_tempty + 8 * buf);
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
       const bool tile_ok = PCED_IN_BOUNDS(tile < ntiles, a.status);
       if (tile_ok) fold_tile(a, tile, etid, wst, wag, wu2);

@@ -15,13 +15,15 @@
 // columns) double buffered and the second (n1) single; the epilogue reads the
 // second one first, so the next tile's MMAs wait for n1 columns of it only.
 //
-// W comes from HBM, H from L2, so they have rings of their own: four stages of
+// W comes from HBM, H from L2, so they have rings of their own: five stages of
 // H, and W in the rest of shared memory (one ring of both, with three stages:
-// 268 against 264 us a call at S = 272; two stages of H: 312).
+// 268 against 264 us a call at S = 272; two stages of H: 312, four: 273 against
+// 265 on another box).  An epilogue warp gives its columns back as soon as they
+// are in its registers (265 -> 257 us).
 //
 // Measured (pced_lm_head_logprobs, d = 4096, V = 128256; one CTA per tile ->
-// pairs): S = 272 370 -> 266 us, S = 384 509 -> 345, S = 512 583 -> 462; in a
-// decode step of 272 sequences 358 -> 218 us.  About half of that came from
+// pairs): S = 272 370 -> 257 us, S = 384 509 -> 345, S = 512 583 -> 462; in a
+// decode step of 272 sequences 358 -> 207 us.  About half of that came from
 // issuing MMAs and copies in warp-uniform code (elect_one in common.cuh), which
 // lm_head.cu has too: with it one CTA per tile is as fast up to 128 rows (192
 // us), 207 against 205 us at 160 and 254 against 239 at 256.
@@ -252,21 +254,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
       const uint32_t b0 = dbl ? acc & 1u : 0u;
       const uint32_t trow = tmem_base + ((uint32_t)(32 * q) << 16);
       auto tcol = [&](int c) { return trow + (c < n0 ? b0 * n0 + c : col1 + (c - n0)); };
-      auto block = [&](int c0) {
-        float z_am = 0.f;
-        if (a.mode == 1 && c0 % n1 != 0) z_am = tmem_ld1(tcol(c0 - c0 % n1));  // the open query's amateur logit
-        epi_block<32>(a, tcol(c0), c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am);
-      };
-      if (nc1) {
-        for (int kb = half; kb < nb1; kb += 2) block(n0 + 32 * kb);
+      // a chunk's columns are free for the next tile's MMAs once this warp's
+      // last ones of them are in its registers
+      auto release = [&](uint32_t bar) {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(tempty1);
-      }
-      for (int kb = (nb1 & 1) ? 1 - half : half; kb < nb0; kb += 2) block(32 * kb);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tempty0 + 8 * b0);
+        if (lane == 0) mbar_arrive_cluster(bar);
+      };
+      auto blocks = [&](int cbase, int kb0, int nb, uint32_t bar) {
+        if (kb0 >= nb) release(bar);
+        for (int kb = kb0; kb < nb; kb += 2) {
+          const int c0 = cbase + 32 * kb;
+          float z_am = 0.f;
+          if (a.mode == 1 && c0 % n1 != 0) z_am = tmem_ld1(tcol(c0 - c0 % n1));  // the open query's amateur logit
+          epi_block<32>(a, tcol(c0), c0, v, valid, lane, q, wbc, wst, wag, wu2, ccoef, cmask, z_am, [&]() {
+            if (kb + 2 >= nb) release(bar);
+          });
+        }
+      };
+      if (nc1) blocks(n0, half, nb1, tempty1);
+      blocks(0, (nb1 & 1) ? 1 - half : half, nb0, tempty0 + 8 * b0);
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
       if (tile < a.ntiles) fold_tile(a, tile, etid, wst, wag, wu2);  // the last pair's second half may hold no rows
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
