@@ -324,6 +324,57 @@ __device__ __forceinline__ void load_merged(const float* ms, const float* ls, co
   mx = M;
 }
 
+// Merges the segment that begins in CTA c of the split kernel and goes on past
+// it (plan; none: nothing): records 2c + 1, 2(c + 1), 2(c + 2), ...  Thread tid
+// holds outputs 4 tid .. 4 tid + 3; the records arrive CMB_BATCH at a time.
+constexpr int CMB_THREADS = ATT_MAX_G * 128 / 4;
+constexpr int CMB_BATCH = 4;
+static_assert(CMB_THREADS == ATT_CT, "the split kernel's consumers can merge");
+
+__device__ __forceinline__ void combine_segment(int c, int2 plan, int32_t Hq, int32_t Hkv, int32_t G, int32_t D,
+                                                const float* rec_o, const float2* rec_ml, float* out) {
+  const int tid = threadIdx.x, GD = G * D;
+  if (plan.y < 2 || 4 * tid >= GD) return;
+  const int hh = 4 * tid / D;
+  float mx = -INFINITY, lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int i0 = 0; i0 < plan.y; i0 += CMB_BATCH) {
+    float2 ml[CMB_BATCH];
+    float4 o[CMB_BATCH];
+#pragma unroll
+    for (int q = 0; q < CMB_BATCH; ++q) {
+      const int i = i0 + q;
+      ml[q] = make_float2(-INFINITY, 0.f);
+      o[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i >= plan.y) continue;
+      const int64_t slot = i == 0 ? 2 * (int64_t)c + 1 : 2 * ((int64_t)c + i);
+      ml[q] = __ldcg(rec_ml + slot * G + hh);
+      o[q] = __ldcg(reinterpret_cast<const float4*>(rec_o + slot * GD + 4 * tid));
+    }
+    float M = mx;
+#pragma unroll
+    for (int q = 0; q < CMB_BATCH; ++q) M = fmaxf(M, ml[q].x);
+    const float f = mx == -INFINITY ? 0.f : exp2f(mx - M);
+    lsum *= f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] *= f;
+#pragma unroll
+    for (int q = 0; q < CMB_BATCH; ++q) {
+      const float e = ml[q].x == -INFINITY ? 0.f : exp2f(ml[q].x - M);
+      acc[0] += o[q].x * e;
+      acc[1] += o[q].y * e;
+      acc[2] += o[q].z * e;
+      acc[3] += o[q].w * e;
+      lsum += ml[q].y * e;
+    }
+    mx = M;
+  }
+  const int s = plan.x / Hkv, h = plan.x - s * Hkv;
+  const float w = 1.f / lsum;
+  float* op = out + (int64_t)s * Hq * D + (int64_t)h * GD + 4 * tid;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) op[j] = mx == -INFINITY ? 0.f : acc[j] * w;
+}
+
 // =================================================================== one layer
 // What bounds it: HBM once a CTA has tens of tiles, the serial chain around
 // them below that (lengths, offsets, first tile, last tile, merge).  The
@@ -518,59 +569,23 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     if (pc.k0 == 0)  // its last key lies (p - 1 + the keys left) positions on
       plan = make_int2(pc.s * a.Hkv + pc.h, (int)(udiv_pos(p - 1 + (len - pc.k1), per) - blockIdx.x) + 1);
   }
-  if (tid == 0) a.plan[blockIdx.x] = plan;
+  if (a.fused) {
+    // all CTAs are one cluster: the records are there for all of them
+    asm volatile(
+        "barrier.cluster.arrive.release;\n\t"
+        "barrier.cluster.wait.acquire;" ::
+            : "memory");
+    combine_segment(blockIdx.x, plan, a.Hq, a.Hkv, G, D, a.rec_o, a.rec_ml, a.out);
+  } else if (tid == 0) {
+    a.plan[blockIdx.x] = plan;
+  }
 }
 
-// CTA c merges the segment that begins in CTA c of the split kernel and goes on
-// past it (if there is one): records 2c + 1, 2(c + 1), 2(c + 2), ...  Thread
-// tid holds outputs 4 tid .. 4 tid + 3; the records arrive CMB_BATCH at a time.
-constexpr int CMB_THREADS = ATT_MAX_G * 128 / 4;
-constexpr int CMB_BATCH = 4;
-
+// The records' merge after a split launch of more CTAs than a cluster holds.
 __global__ void __launch_bounds__(CMB_THREADS) att_combine_kernel(CombineArgs a) {
-  const int c = blockIdx.x, tid = threadIdx.x, GD = a.G * a.D;
   pdl_launch_dependents();
   pdl_wait();
-  const int2 plan = a.plan[c];
-  if (plan.y < 2 || 4 * tid >= GD) return;
-  const int hh = 4 * tid / a.D;
-  float mx = -INFINITY, lsum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int i0 = 0; i0 < plan.y; i0 += CMB_BATCH) {
-    float2 ml[CMB_BATCH];
-    float4 o[CMB_BATCH];
-#pragma unroll
-    for (int q = 0; q < CMB_BATCH; ++q) {
-      const int i = i0 + q;
-      ml[q] = make_float2(-INFINITY, 0.f);
-      o[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i >= plan.y) continue;
-      const int64_t slot = i == 0 ? 2 * (int64_t)c + 1 : 2 * ((int64_t)c + i);
-      ml[q] = a.rec_ml[slot * a.G + hh];
-      o[q] = *reinterpret_cast<const float4*>(a.rec_o + slot * GD + 4 * tid);
-    }
-    float M = mx;
-#pragma unroll
-    for (int q = 0; q < CMB_BATCH; ++q) M = fmaxf(M, ml[q].x);
-    const float f = mx == -INFINITY ? 0.f : exp2f(mx - M);
-    lsum *= f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[j] *= f;
-#pragma unroll
-    for (int q = 0; q < CMB_BATCH; ++q) {
-      const float e = ml[q].x == -INFINITY ? 0.f : exp2f(ml[q].x - M);
-      acc[0] += o[q].x * e;
-      acc[1] += o[q].y * e;
-      acc[2] += o[q].z * e;
-      acc[3] += o[q].w * e;
-      lsum += ml[q].y * e;
-    }
-    mx = M;
-  }
-  const int s = plan.x / a.Hkv, h = plan.x - s * a.Hkv;
-  const float w = 1.f / lsum;
-  float* op = a.out + (int64_t)s * a.Hq * a.D + (int64_t)h * GD + 4 * tid;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) op[j] = mx == -INFINITY ? 0.f : acc[j] * w;
+  combine_segment(blockIdx.x, a.plan[blockIdx.x], a.Hq, a.Hkv, a.G, a.D, a.rec_o, a.rec_ml, a.out);
 }
 
 // ============================================================ whole step
@@ -1632,13 +1647,30 @@ static cudaError_t launch_split(const CUtensorMap& kmap, const CUtensorMap& vmap
   static bool configured[64];
   cudaError_t e = set_smem_once(att_split_kernel<D, PK>, AttCfg<D>::SMEM, configured);
   if (e != cudaSuccess) return e;
-  return pced_host::launch_pdl(att_split_kernel<D, PK>, dim3(ctas), ATT_THREADS, AttCfg<D>::SMEM, stream, kmap, vmap,
-                               a);
+  return pced_host::launch_cluster(att_split_kernel<D, PK>, dim3(ctas), a.fused ? ctas : 0, ATT_THREADS,
+                                   AttCfg<D>::SMEM, stream, true, kmap, vmap, a);
+}
+
+// Few keys in few segments: one cluster of up to eight CTAs, which merge their
+// records themselves, instead of a CTA for every 128 keys and a second launch.
+// A call among others, two launches / one: 1478 keys, D = 64, 6 segments 7.5 /
+// 6.5 us; 3112 keys, D = 128, 24 segments 9.3 / 8.1; 3986 keys, G = 8, D = 64 9.0 /
+// 8.0; but 1956 keys, G = 7, D = 128 8.4 / 9.2 (972 keys 7.9 / 6.9), 4010 keys in 38
+// segments 8.7 / 11.3 and 6530 keys 7.9 / 10.9.
+static bool att_one_cluster(int32_t S, int32_t Hkv, int32_t G, int32_t D, int64_t keys) {
+  return (int64_t)S * Hkv <= 24 && keys <= (G * D <= 512 ? 4096 : 1024);
+}
+// CTAs of a cluster for few keys: a power of two up to 8, a CTA for every 128 keys
+static int att_cluster(int64_t keys) {
+  int n = 1;
+  while (n < 8 && (int64_t)n * 128 < keys) n *= 2;
+  return n;
 }
 
 cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, AttArgs a, int64_t total_cap_keys,
                              void* scratch, cudaStream_t stream) {
-  int ctas = att_grid(total_cap_keys, 128);
+  a.fused = att_one_cluster(a.S, a.Hkv, a.G, D, total_cap_keys);
+  int ctas = a.fused ? att_cluster(total_cap_keys) : att_grid(total_cap_keys, 128);
   if (ctas > ATT_SPLIT_CTAS) ctas = ATT_SPLIT_CTAS;
   pced_host::Carver cv(scratch);
   a.rec_o = cv.take<float>((size_t)2 * ctas * a.G * D);
@@ -1650,7 +1682,7 @@ cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& 
     e = pk ? launch_split<128, true>(kmap, vmap, a, ctas, stream) : launch_split<128, false>(kmap, vmap, a, ctas, stream);
   else if (D == 64)
     e = pk ? launch_split<64, true>(kmap, vmap, a, ctas, stream) : launch_split<64, false>(kmap, vmap, a, ctas, stream);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || a.fused) return e;
   const CombineArgs c = {a.Hq, a.Hkv, a.G, D, a.rec_o, a.rec_ml, a.plan, a.out};
   return pced_host::launch_pdl(att_combine_kernel, dim3(ctas), CMB_THREADS, 0, stream, c);
 }

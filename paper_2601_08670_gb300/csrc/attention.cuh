@@ -39,10 +39,11 @@ struct AttArgs {
   float* rec_o;               // [2 * CTAs][G][D] unnormalised partial outputs
   float2* rec_ml;             // [2 * CTAs][G] (running max in log2 units, sum of exp2)
   int2* plan;                 // [CTAs] (s * Hkv + h, records), records < 2: none
+  bool fused;                 // the CTAs are one cluster and merge their records themselves
   int* status;
 };
 
-// Merges the records: CTA c the segment of plan[c].
+// Merges the records (not of a fused launch): CTA c the segment of plan[c].
 struct CombineArgs {
   int32_t Hq, Hkv, G, D;
   const float* rec_o;

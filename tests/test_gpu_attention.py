@@ -99,3 +99,18 @@ def test_bad_length_sets_device_status_without_faulting(cuda_ok):
 ])
 def test_records_and_whole_segments(cuda_ok, lens, Hq, Hkv, D):
     assert run_case(lens, Hq=Hq, Hkv=Hkv, D=D, extra=0, seed=5) < 1e-4
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,D,extra", [
+    ([1], 1, 1, 64, 0),             # one CTA, one key
+    ([128], 4, 1, 128, 0),          # one CTA, full
+    ([129], 4, 1, 128, 0),          # two CTAs, one segment
+    ([1000, 24], 8, 1, 64, 0),      # eight CTAs, one segment over almost all of them (1024 keys)
+    ([200, 1, 311], 8, 8, 128, 0),  # 24 segments: the most a single cluster takes
+    ([200, 1, 311, 1], 8, 8, 128, 0),  # 32 segments: two launches
+    ([2048], 4, 2, 128, 0), ([2049], 4, 2, 128, 0),    # at and past 4096 keys
+    ([256], 28, 4, 128, 0), ([257], 28, 4, 128, 0),    # seven heads per kv-head: at and past 1024 keys
+    ([5, 7], 4, 2, 64, 900),        # mostly empty CTAs: the capacity sizes the grid
+])
+def test_one_cluster_and_two_launches(cuda_ok, lens, Hq, Hkv, D, extra):
+    assert run_case(lens, Hq=Hq, Hkv=Hkv, D=D, extra=extra, seed=8) < 1e-4
