@@ -382,10 +382,10 @@ __device__ __forceinline__ void combine_segment(int c, int2 plan, int32_t Hq, in
 // before the partition is known, so no piece waits for its own; a segment that
 // a CTA holds whole is normalised and written by it, and only the segments cut
 // by a CTA boundary (at most one per CTA) leave records for the second kernel,
-// which is resident by then (programmatic launch).  Measured, a call among
-// others: 9 x 2081 keys, 8 kv-heads, D = 128 (68.5 MB): 32.2 -> 18.0 us; 17 x
-// 4129 keys, 4 kv-heads, 7 heads each (136 MB): 50.1 -> 29.2 us; 272 ragged
-// sequences (1.27 GB): 208.9 -> 190.4 us (98 % of the copy bandwidth).  Before,
+// whose launch overlaps the first one's end (programmatic launch).  Measured, a call among
+// others: 9 x 2081 keys, 8 kv-heads, D = 128 (68.5 MB): 32.2 -> 16.8 us; 17 x
+// 4129 keys, 4 kv-heads, 7 heads each (136 MB): 49.4 -> 27.5 us; 272 ragged
+// sequences (1.27 GB): 206.9 -> 187.7 us (99.6 % of the copy bandwidth).  Before,
 // a combine CTA per segment read the whole partition and its records in four
 // dependent round trips (8.9-11.3 us) after the split kernel had ended.
 template <int D, bool PK>
@@ -424,7 +424,6 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     tma_prefetch_desc(&kmap);
     tma_prefetch_desc(&vmap);
   }
-  pdl_launch_dependents();
   pdl_wait();
   // live lengths, clamped into [1, cap] (out-of-range lengths are flagged)
   for (int i = tid; i < S; i += ATT_THREADS) {
@@ -579,11 +578,14 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
   } else if (tid == 0) {
     a.plan[blockIdx.x] = plan;
   }
+  // the next kernel's CTAs come now (had they come at the start and waited
+  // beside this one, 9 x 2081 keys would take 17.0 us instead of 16.4, 17 x 4129
+  // keys 28.1 instead of 27.0)
+  pdl_launch_dependents();
 }
 
 // The records' merge after a split launch of more CTAs than a cluster holds.
 __global__ void __launch_bounds__(CMB_THREADS) att_combine_kernel(CombineArgs a) {
-  pdl_launch_dependents();
   pdl_wait();
   combine_segment(blockIdx.x, a.plan[blockIdx.x], a.Hq, a.Hkv, a.G, a.D, a.rec_o, a.rec_ml, a.out);
 }
