@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
     tma_prefetch_desc(&wmap);
     tma_prefetch_desc(&hmap);
   }
-  pdl_launch_dependents();
+  if (a.mode == 1) pdl_launch_dependents();
   if (warp == 1) {
     tmem_alloc(smem_u32(tmem_slot), a.tmem_cols);
     tmem_relinquish();
@@ -388,6 +388,11 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
+  // the log-softmax or aggregation kernels come at the end: beside this one
+  // their CTAs only wait (S = 272 252 -> 247 us a call, S = 33, d = 1024, V = 50000
+  // 29.1 -> 27.4); the selection's cluster, which starts later, comes early
+  // (the 9-row step 538 us, 543 with a late one)
+  if (a.mode == 0) pdl_launch_dependents();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, a.tmem_cols);

@@ -18,7 +18,7 @@
 // W comes from HBM, H from L2, so they have rings of their own: five stages of
 // H, and W in the rest of shared memory (one ring of both, with three stages:
 // 268 against 264 us a call at S = 272; two stages of H: 312, four: 273 against
-// 265 on another box).  An epilogue warp gives its columns back as soon as they
+// 265 with five).  An epilogue warp gives its columns back as soon as they
 // are in its registers (265 -> 257 us).
 //
 // Measured (pced_lm_head_logprobs, d = 4096, V = 128256; one CTA per tile ->
@@ -89,7 +89,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
     tma_prefetch_desc(&hmap0);
     if (nc1) tma_prefetch_desc(&hmap1);
   }
-  pdl_launch_dependents();
+  if (a.mode == 1) pdl_launch_dependents();
   if (warp == 1) tmem_alloc_pair(smem_u32(tmem_slot), 512);
   if (a.mode == 1) column_tables(a, tid, ccoef, cmask);
   tc_fence_before();
@@ -282,6 +282,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();  // neither CTA's shared memory, barriers or TMEM is used by the other any more
+  if (a.mode == 0) pdl_launch_dependents();  // see lm_head.cu
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem_base, 512);
