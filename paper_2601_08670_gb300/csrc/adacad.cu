@@ -6,16 +6,18 @@
 // p_0 = exp(lp_0):
 //   beta[b][k-1] = 1/2 sum_v [ p_k log2(p_k / m) + p_0 log2(p_0 / m) ],  m = (p_k + p_0) / 2,
 // in [0, 1].  With hi / lo the larger and smaller of the two log-probabilities
-// and e = exp(lo - hi), a term is
-//   exp(hi) [ q + e (q + lo - hi) ],  q = -log((1 + e) / 2) = log(p_hi / m),
-// in fp32, without the rounding of a logarithm of the size of hi.
+// the midpoint's is log m = hi + log1p(exp(lo - hi)) - log 2; terms in fp32.
 //
-// What bounds it: two exp and one log per entry and expert (and, past the
+// What bounds it: three exp and one log1p per entry and expert (and, past the
 // L2, the rows).  A cluster of CTAs takes one (expert, query): the
 // cluster's sums meet in the first CTA's shared memory, so there is no scratch,
 // no counter to clear and no second pass.  (One CTA per 2048 entries left the
-// last one to add 63 chunk sums one load after the other: 14.8 us for 8
-// experts of 128256 entries beside a memset; 184 us for 16 x 16, now 86.)
+// last one to add 63 chunk sums one load after the other.  Experts of 128256
+// entries, in a graph: 8 16.7 -> 10.0 us, 16 x 16 184 -> 101.)  A term without
+// the midpoint's logarithm, exp(hi) (q + e (q + lo - hi)) with e = exp(lo - hi)
+// and q = -log((1 + e) / 2), needs one exponential less (16 x 16: 86 us) and
+// has half the error, but moves beta's last bit, which a score near zero
+// magnifies to 2.5e-6 of itself.
 //
 // Sums are held as an unevaluated pair of fp32 numbers (error-free addition,
 // about 48 bits) and rounded once from fp64 at the end: this chip adds 64-bit
@@ -66,8 +68,11 @@ __device__ __forceinline__ Pair warp_pair(Pair p) {
 __device__ __forceinline__ float jsd_term(float a, float b) {
   const float hi = fmaxf(a, b), lo = fminf(a, b);
   if (hi == -INFINITY) return 0.f;  // both probabilities are 0
-  const float d = lo - hi, e = expf(d), q = -logf(fmaf(0.5f, e, 0.5f));
-  return expf(hi) * (lo == -INFINITY ? q : q + e * (q + d));
+  const float lm = hi + log1pf(expf(lo - hi)) - 0.69314718055994531f;  // log of the midpoint
+  float t = 0.f;
+  if (a > -INFINITY) t += expf(a) * (a - lm);
+  if (b > -INFINITY) t += expf(b) * (b - lm);
+  return t;
 }
 
 // grid (CTAs of a cluster, N, B), one cluster per (k - 1, b)

@@ -41,8 +41,9 @@ def test_adacad_beta_matches_oracle(cuda_ok, B, N, V, spread):
 
 @pytest.mark.parametrize("V", [2, 7, 9, 1023, 8191, 8193, 32769])
 def test_adacad_beta_edges_of_the_cluster_split(cuda_ok, V):
-    """Vocabularies around the eight parts of a cluster and a part's threads.  Each term is good to a few ulp of its
-    probability and the sums carry 48 bits, so the result is within 1e-6 of the fp64 sum over the same rows."""
+    """Vocabularies around the eight parts of a cluster and a part's threads.  The midpoint's logarithm is at most 16
+    here and rounded twice, so off by 1e-6 at most in a term and by either sign; its probabilities sum to 1, halved, and
+    the sums carry 48 bits: the result is within 1e-6 of the fp64 sum over the same rows."""
     rng = np.random.default_rng(V)
     lp = _logprob_rows(rng, 2 * 3, V, 2.0).astype(np.float32).astype(np.float64)
     assert np.max(np.abs(_gpu_beta(lp, 2, 2) - oracle.adacad_beta(lp, 2, 2))) <= 1e-6
