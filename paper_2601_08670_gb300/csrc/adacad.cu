@@ -82,8 +82,7 @@ __global__ void __launch_bounds__(ADA_THREADS)
   const int rank = blockIdx.x, nc = gridDim.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
   __shared__ Pair wsum[ADA_THREADS / 32], csum[ROW_CLUSTER];
   cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
-  pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait();  // dependents are launched when this ends: select.cu has the figures
   if (reset_ctr && rank == 0 && k == 1 && b == 0 && tid == 0) *reset_ctr = 0;
   const float* l0 = lp + (int64_t)b * (N + 1) * V;
   const float* lk = l0 + (int64_t)k * V;

@@ -14,7 +14,11 @@
 // rows.  Now a thread has SEL_TOK tokens of SEL_ROWS experts in flight, four
 // CTAs share a chunk (their bests meet in the first one's shared memory, so
 // the workspace still holds one record per SEL_CHUNK tokens), and the second
-// kernel is resident before the first one ends (programmatic launch).
+// kernel's launch is set up beside the first (programmatic launch).  Neither
+// this kernel nor adacad.cu's triggers its dependents early: CTAs that only
+// wait would hold the slots of its own later ones (beta, select and relevance
+// in a graph, us: 33 rows of V = 128256 34.4 -> 25.1, 9 rows 16.3 -> 15.7,
+// 4 x 9 rows of V = 50000 18.8 -> 16.3).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -59,7 +63,6 @@ __global__ void __cluster_dims__(SEL_CLUSTER, 1, 1) __launch_bounds__(SEL_THREAD
   __shared__ float bt[SEL_MAX_N], bias[SEL_MAX_N];
   __shared__ Cand wbest[SEL_THREADS / 32], cbest[SEL_CLUSTER];
   cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
-  pdl_launch_dependents();
   pdl_wait();
   for (int k = tid; k < N; k += SEL_THREADS) {
     bt[k] = beta[b * N + k];
