@@ -520,7 +520,12 @@ cudaError_t lm_lse_finalize_launch(float* logits, const float2* rec_stats, float
 // in flight together and their maximum is the thread's own first, so one pass
 // does.  Measured (one CTA per row with an arrival counter -> this): 9 rows
 // 12.4 -> 10.1 us, 33 rows 17.4 -> 10.6, 129 rows 35 -> 21, 16 x 17 rows 19.0 ->
-// 13.2, 3 rows of d = 512 9.3 -> 8.4.
+// 13.2, 3 rows of d = 512 9.3 -> 8.4.  A row's warps meet in the lanes of its
+// first one (each receiver used to add the sixteen results one after another),
+// and beta and r are loaded while the cluster meets: a step of 3 rows and one
+// layer 37.7 -> 36.7 us, of 9 rows and 32 layers 528.8 -> 527.6.  Loading them
+// beside the records cost 16 x 17 rows 2 us; an L2 prefetch of each candidate's
+// row of W gained nothing.
 constexpr int SEL_R_THREADS = 512;
 constexpr int SEL_R_WARPS = SEL_R_THREADS / 32;
 constexpr int SEL_R_CLUSTER = 8;  // most CTAs per query
@@ -601,31 +606,45 @@ __global__ void __launch_bounds__(SEL_R_THREADS) select_from_records_kernel(Sele
     __syncthreads();
     if (!started) cluster.barrier_wait();
     started = true;
-    if (on && gt < nc) {  // thread gt writes the row's results to CTA gt
-      float M = -INFINITY, L = 0.f;
-      bu = b2 = -INFINITY;
-      bv = 0x7fffffff;
-      for (int w = grp * wpr; w < (grp + 1) * wpr; ++w) {
-        M = fmaxf(M, sm[w]);
-        top2_merge(bu, bv, b2, sv[w], si[w], sv2[w]);
+    if (on && gt < 32) {  // the row's first warp: lane w takes warp w's results
+      const int w = grp * wpr + lane;
+      const bool in = lane < wpr;
+      m = in ? sm[w] : -INFINITY;
+      bu = in ? sv[w] : -INFINITY;
+      b2 = in ? sv2[w] : -INFINITY;
+      bv = in ? si[w] : 0x7fffffff;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float r1 = __shfl_xor_sync(0xffffffffu, bu, o), r2 = __shfl_xor_sync(0xffffffffu, b2, o);
+        const int rt = __shfl_xor_sync(0xffffffffu, bv, o);
+        top2_merge(bu, bv, b2, r1, rt, r2);
       }
-      for (int w = grp * wpr; w < (grp + 1) * wpr; ++w) L += sm[w] == -INFINITY ? su[w] : su[w] * expf(sm[w] - M);
+      const float M = warp_max(m), e = !in ? 0.f : m == -INFINITY ? su[w] : su[w] * expf(m - M);
+      float L = 0.f;
+      for (int i = 0; i < wpr; ++i) L += __shfl_sync(0xffffffffu, e, i);  // the warps in order
       L = M + logf(L);
-      cluster.map_shared_rank(row_L, gt)[j] = L;
-      cluster.map_shared_rank(row_u, gt)[j] = bu;
-      cluster.map_shared_rank(row_u2, gt)[j] = b2;
-      cluster.map_shared_rank(row_tok, gt)[j] = bv;
-      if (gt == 0 && a.lse_out) a.lse_out[s] = L;
+      if (lane < nc) {  // lane c writes to CTA c
+        cluster.map_shared_rank(row_L, lane)[j] = L;
+        cluster.map_shared_rank(row_u, lane)[j] = bu;
+        cluster.map_shared_rank(row_u2, lane)[j] = b2;
+        cluster.map_shared_rank(row_tok, lane)[j] = bv;
+        if (lane == 0 && a.lse_out) a.lse_out[s] = L;
+      }
     }
     if (q0 + rf < rows) __syncthreads();  // the partial results are used again
   }
-  cluster.sync();
+  cluster.barrier_arrive();
+  // warp 0's first experts' beta and relevance arrive while the cluster meets
+  const float beta0 = warp == 0 && lane < N ? a.beta[b * N + lane] : 0.f;
+  const float r0 = warp == 0 && lane < N ? a.r[b * N + lane] : 1.f;
+  cluster.barrier_wait();
   float bs = -INFINITY;
   int bt = 0x7fffffff, bk = 0x7fffffff;
-  // Eq. 2's per-expert constant
+  // Eq. 2's per-expert constant (warp 0, k = lane + 32 i)
+  auto beta_of = [&](int k) { return k < 32 ? beta0 : a.beta[b * N + k]; };
   auto bias = [&](int k) {
-    const float btk = a.beta[b * N + k];
-    const float rr = fminf(fmaxf(a.r[b * N + k], 1e-8f), 1.0f);
+    const float btk = beta_of(k);
+    const float rr = fminf(fmaxf(k < 32 ? r0 : a.r[b * N + k], 1e-8f), 1.0f);
     return (a.raw_logits ? 0.f : -(1.f + btk) * row_L[1 + k] + btk * row_L[0]) + a.gamma * logf(rr);
   };
   if (warp == 0) {
@@ -711,7 +730,7 @@ __global__ void __launch_bounds__(SEL_R_THREADS) select_from_records_kernel(Sele
       // token gap: the best score at another token, over all experts
       float other = -INFINITY, se_best = -INFINITY, se_other = -INFINITY;
       for (int k = lane; k < N; k += 32) {
-        const float c = bias(k), btk = a.beta[b * N + k];
+        const float c = bias(k), btk = beta_of(k);
         other = fmaxf(other, (row_tok[1 + k] != bt ? row_u[1 + k] : row_u2[1 + k]) + c);
         // expert gap: every expert's score at the chosen token, from the recomputed logits
         const float se = (1.f + btk) * zy[1 + k] - btk * zy[0] + c;
