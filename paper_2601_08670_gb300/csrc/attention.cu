@@ -1618,14 +1618,10 @@ int att_step_seg_cost(int D) { return env_int("PCED_ATT_SEGCOST", 512, 0, 1 << 2
 int att_step_pf_tiles() { return env_int("PCED_ATT_PF", 6, 0, 64); }
 // Two groups, the second of which streams while the first one's layer dependency
 // resolves (eight layers of 9 sequences of 2080 rows: 120 us against 137 with
-// one); one group where there are many more segments than CTAs, so that few
-// are split, CTAs hardly wait for one another and the second group's pieces
-// only cost (two layers of 272 sequences around 1184 rows: 449 us against 469,
-// of 65 sequences of 544 rows 77 against 82; equal within 1 % at 1.7 segments
-// per CTA).
-int att_step_groups(int32_t S, int32_t Hkv, int ctas) {
-  return env_int("PCED_ATT_GROUPS", (int64_t)S * Hkv > 3 * (int64_t)ctas ? 1 : 2, 1, ATT_MAX_GROUPS);
-}
+// one).  Two also where segments are many more than CTAs, so that few are split
+// and one group would do: another number of groups moves the cuts, and with them
+// the order of the sums and some bf16 roundings of every later layer.
+int att_step_groups() { return env_int("PCED_ATT_GROUPS", 2, 1, ATT_MAX_GROUPS); }
 int att_step_seg_lead(int seg_cost) { return env_int("PCED_ATT_LEAD", seg_cost / 2, 0, seg_cost); }
 
 // cudaFuncSetAttribute once per kernel and device

@@ -252,8 +252,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   at.rms_eps = p->rms_eps;
   at.seg_cost = att_step_seg_cost(dm.D);
   at.pf_tiles = att_step_pf_tiles();
-  const int att_ctas = att_grid(p->total_cap * dm.Hkv, 256);
-  at.groups = att_step_groups(S, dm.Hkv, att_ctas);
+  at.groups = att_step_groups();
   at.seg_lead = att_step_seg_lead(at.seg_cost);
   if (paged) {
     // whole tiles: with every extent, lead and CTA share a multiple of the
@@ -290,7 +289,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   at.status = W.status;
   at.wait_ns = p->wait_limit_ns ? p->wait_limit_ns : kWaitLimitNs;
   ranges.next("attention");
-  e = att_step_launch(dm.D, kmap, vmap, at, att_ctas, s);
+  e = att_step_launch(dm.D, kmap, vmap, at, att_grid(p->total_cap * dm.Hkv, 256), s);
   if (e == cudaSuccess) e = mark();
   if (e != cudaSuccess) return cuda_status(e, "attention launch");
 

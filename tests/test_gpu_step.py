@@ -204,6 +204,27 @@ def test_llama8_sequence_groups(cuda_ok, monkeypatch, groups):
     run_parity("llama8", 2, min_ram_gb=8)
 
 
+def test_two_sequence_groups_at_every_batch_size(cuda_ok, monkeypatch):
+    # 65 sequences of 8 kv heads, several times as many segments as CTAs: the
+    # default is the two-group partition here too, so every sum keeps its order
+    # and a batched step its hidden states and appended rows, bit for bit
+    import paper_2601_08670_gb300 as pced
+    w = synth.get("llama8", L=3, B=5, N=12, V=1000, doc_len=("uniform", 100, 500), steps=2)
+    assert w.S * w.Hkv > 3 * 152
+    out = []
+    for groups in (None, "2"):
+        if groups:
+            monkeypatch.setenv("PCED_ATT_GROUPS", groups)
+        dec, t = make_decoder(w, torch.device("cuda"))
+        for _ in range(2):
+            dec.step()
+        torch.cuda.synchronize()
+        assert dec.status() == 0
+        out.append((bf16_bits(dec.hidden), bf16_bits(t["k_cache"]), bf16_bits(t["v_cache"])))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
 def test_qwen_flat_full_size(cuda_ok):
     run_parity("qwen_flat", 6, min_ram_gb=10)
 
