@@ -177,6 +177,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
       if (++h == hst_n) h = 0;
       if (++hw == wst_n) hw = 0;
     }
+    // CTA 0's commits arrive on the barriers of both CTAs, and an arrival must
+    // not find its CTA gone: both producers see the last commit of every stage,
+    // and CTA 1's the one after the last MMA too, which nothing else waits for
+    // there (CTA 0's MMA warp does; the epilogues wait for the tiles' commits)
+    for (uint32_t j = nw > wst_n ? nw - wst_n : 0; ok && j < nw; ++j)
+      ok = mbar_wait_warp(bar_empty + 8 * (j % wst_n), (j / wst_n) & 1u, a.status);
+    if (rank == 1) mbar_wait_warp(bar_drain, 0, a.status);
     if (!ok) {
       // let the copies in flight land: a thousand times a copy's latency
       const uint64_t t0 = globaltimer_ns();
@@ -281,7 +288,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();  // neither CTA's shared memory, barriers or TMEM is used by the other any more
+  // neither CTA's shared memory, barriers or TMEM is used by the other any more:
+  // both have seen every arrival on a barrier of theirs (above)
+  cluster_sync_all();
   if (a.mode == 0) pdl_launch_dependents();  // see lm_head.cu
   if (warp == 1) {
     tc_fence_after();

@@ -168,6 +168,21 @@ def test_tiny_ragged_vocabularies(cuda_ok, V):
     run_parity("tiny", 3, V=V)
 
 
+@pytest.mark.parametrize("B,N,V", [
+    (7, 22, 1128),       # 161 sequences: the fewest that take CTA pairs; 9 vocabulary tiles, so half of the last pair's
+                         # rows lie past the vocabulary
+    (8, 23, 300),        # 192 sequences, 2 pairs for 3 tiles: a pair that comes late claims none
+    (1, 192, 100),       # 193 sequences, one pair, half of it without rows
+    (15, 16, 8192 + 77), # 255 sequences: the widest accumulator of one chunk; 33 pairs of tiles
+    (20, 19, 1000),      # 400 sequences: two chunks, neither double buffered
+])
+def test_pairs_of_ctas(cuda_ok, B, N, V):
+    # the fused LM head of more than 160 sequences: queries whose experts lie
+    # across 32-column blocks and chunks, an odd number of vocabulary tiles, and
+    # pairs that end without a tile or just after their last one
+    run_parity("tiny", 4, B=B, N=N, V=V)
+
+
 @pytest.mark.parametrize("Hq,Hkv,D", [(4, 2, 64), (6, 2, 128), (16, 2, 64), (16, 2, 128), (12, 4, 128)])
 def test_tiny_head_shapes(cuda_ok, Hq, Hkv, D):
     # query heads per kv head G = 2, 3, 8, 8, 3 with D = 64 / 128: the packed
