@@ -144,6 +144,15 @@ __device__ __forceinline__ void mbar_arrive_expect_tx_if(uint32_t on, uint32_t b
       "r"(bytes), "r"(on)
       : "memory");
 }
+// bytes of the current phase that no copy will bring, counted as landed
+__device__ __forceinline__ void mbar_complete_tx_if(uint32_t on, uint32_t bar, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %2, 0;\n\t"
+      "@q mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n\t}" ::"r"(bar),
+      "r"(bytes), "r"(on)
+      : "memory");
+}
 // mbar_wait by a whole warp, the same answer in every lane
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* status) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, status));

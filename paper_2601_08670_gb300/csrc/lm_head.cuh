@@ -48,6 +48,23 @@ struct LmArgs {
   int* status;
 };
 
+// The copies of a pair that are still on their way when a producer has given
+// up.  n0, n1: slabs (of W and H) that CTA 0 and CTA 1 have asked for, whose
+// bytes CTA 0's full barriers count; for a slab of its own CTA 0 has arrived on
+// its stage's barrier with the bytes of both.  The two counts differ by at most
+// `stages`: neither asks for slab n before slab n - stages has been consumed.
+// Waits until every copy of both has landed; false if that wait runs out.
+#pragma nv_exec_check_disable  // (the barriers are the device's, or a model of them on the host)
+template <class Ring>
+__host__ __device__ inline bool lm_pair_drain(uint32_t n0, uint32_t n1, uint32_t stages, Ring& ring) {
+  const uint32_t n = n0 > n1 ? n0 : n1;
+  for (uint32_t j = n0; j < n; ++j) ring.expect_one(j % stages);  // CTA 1 alone asked for it: its bytes
+  for (uint32_t j = n1; j < n; ++j) ring.missing_one(j % stages);  // CTA 0 alone did: the other bytes never come
+  for (uint32_t j = n > stages ? n - stages : 0; j < n; ++j)
+    if (!ring.wait(j % stages, (j / stages) & 1u)) return false;
+  return true;
+}
+
 struct LmMaps {
   CUtensorMap w, h[2];  // W tiles; H rows of the N chunks
 };

@@ -37,6 +37,15 @@
 
 namespace pced {
 
+// CTA 0's full barriers for lm_pair_drain (a whole warp, `on` in one lane)
+struct PairFull {
+  uint32_t on, bar, bytes;  // bytes of one CTA's share of a slab
+  int* status;
+  __device__ void expect_one(uint32_t w) { mbar_arrive_expect_tx_if(on, bar + 8 * w, bytes); }
+  __device__ void missing_one(uint32_t w) { mbar_complete_tx_if(on, bar + 8 * w, bytes); }
+  __device__ bool wait(uint32_t w, uint32_t parity) { return mbar_wait_warp(bar + 8 * w, parity, status); }
+};
+
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
     lm_head_pair_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap hmap0,
                         const __grid_constant__ CUtensorMap hmap1, LmArgs a) {
@@ -48,7 +57,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
   const uint32_t b_bytes = (uint32_t)S_pad * 64u;  // this CTA's half of an H slab
   const uint32_t wst_n = a.stages, hst_n = a.hstages;
   // layout: W ring | H ring | full[W stages] | empty[W stages] | tfull[2] | tempty0[2] | tempty1 |
-  //         claim[LM_TRING] | epi | drain | tmem slot, tile ring | scratch
+  //         claim[LM_TRING] | epi | drain | done | tmem slot, CTA 1's slabs, tile ring | scratch
   const uint32_t hbase = base + wst_n * LM_A_BYTES;
   const uint32_t bar_full = hbase + hst_n * b_bytes;
   const uint32_t bar_empty = bar_full + 8 * wst_n;
@@ -58,9 +67,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
   const uint32_t bar_claim = bar_tempty1 + 8;
   const uint32_t bar_epi = bar_claim + 8 * LM_TRING;
   const uint32_t bar_drain = bar_epi + 8;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + (bar_drain + 8 - base));
+  const uint32_t bar_done = bar_drain + 8;  // CTA 0: CTA 1's producer has asked for its last slab
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + (bar_done + 8 - base));
+  uint32_t* peer_slabs = tmem_slot + 1;     // CTA 0: how many that were
   int32_t* tring = reinterpret_cast<int32_t*>(tmem_slot + 4);  // [LM_TRING] claimed tiles
-  float2* wst = reinterpret_cast<float2*>(gbase + ((bar_drain + 8 - base + 16 + 4 * LM_TRING + 15) & ~15u));
+  float2* wst = reinterpret_cast<float2*>(gbase + ((bar_done + 8 - base + 16 + 4 * LM_TRING + 15) & ~15u));
   float2* wag = wst + 4 * S_pad;                           // [4][S_pad] per-warp argmax
   float* wu2 = reinterpret_cast<float*>(wag + 4 * S_pad);  // [4][S_pad] per-warp runner-up
   float2* ccoef = wag + 6 * S_pad;                         // [S_pad] (1 + beta, beta) per column
@@ -82,6 +93,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
     for (int i = 0; i < LM_TRING; ++i) mbar_init(bar_claim + 8 * i, 1);
     mbar_init(bar_epi, LM_EPI_THREADS);
     mbar_init(bar_drain, 1);
+    mbar_init(bar_done, 1);
     mbar_fence_init();
   }
   if (warp == 0 && lane == 0) {
@@ -177,17 +189,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
       if (++h == hst_n) h = 0;
       if (++hw == wst_n) hw = 0;
     }
+    // a producer that gave up leaves whole slabs behind: their H follows their W
+    while (nh < nw) {
+      load_h(h, hw);
+      ++nh;
+      if (++h == hst_n) h = 0;
+      if (++hw == wst_n) hw = 0;
+    }
+    if (rank == 1 && lane == 0) {
+      st_cluster_u32(mapa(smem_u32(peer_slabs), 0), nw);
+      mbar_arrive_cluster(mapa(bar_done, 0));
+    }
     // CTA 0's commits arrive on the barriers of both CTAs, and an arrival must
     // not find its CTA gone: both producers see the last commit of every stage,
     // and CTA 1's the one after the last MMA too, which nothing else waits for
     // there (CTA 0's MMA warp does; the epilogues wait for the tiles' commits)
     for (uint32_t j = nw > wst_n ? nw - wst_n : 0; ok && j < nw; ++j)
       ok = mbar_wait_warp(bar_empty + 8 * (j % wst_n), (j / wst_n) & 1u, a.status);
-    if (rank == 1) mbar_wait_warp(bar_drain, 0, a.status);
-    if (!ok) {
-      // let the copies in flight land: a thousand times a copy's latency
-      const uint64_t t0 = globaltimer_ns();
-      while (globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
+    if (rank == 1) {
+      mbar_wait_warp(bar_drain, 0, a.status);
+    } else {
+      // CTA 1 may be at a wait that runs out one limit later; then both CTAs'
+      // copies land before either leaves the cluster barrier below (with every
+      // stage's last commit seen there are none)
+      const bool met = mbar_wait_cluster(bar_done, 0, a.status) || mbar_wait_cluster(bar_done, 0, a.status);
+      const uint32_t n1 = met ? *(volatile uint32_t*)peer_slabs : nw;
+      PairFull full{on, bar_full, LM_A_BYTES + b_bytes, a.status};
+      if (!ok) lm_pair_drain(nw, __shfl_sync(0xffffffffu, n1, 0), wst_n, full);
     }
     __syncwarp();
   } else if (warp == 1) {
