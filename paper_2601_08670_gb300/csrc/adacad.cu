@@ -75,9 +75,12 @@ __device__ __forceinline__ float jsd_term(float a, float b) {
   return t;
 }
 
-// grid (CTAs of a cluster, N, B), one cluster per (k - 1, b)
+// grid (CTAs of a cluster, N, B), one cluster per (k - 1, b).  lp is a plain
+// pointer: the launch before may still rewrite the rows when this one starts
+// (the log-softmax pass does, in place), so its loads must not become
+// non-coherent ones, which const __restrict__ allows.
 __global__ void __launch_bounds__(ADA_THREADS)
-    adacad_beta_kernel(const float* __restrict__ lp, int32_t N, int32_t V, float* beta, int* reset_ctr) {
+    adacad_beta_kernel(const float* lp, int32_t N, int32_t V, float* beta, int* reset_ctr) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = blockIdx.x, nc = gridDim.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
   __shared__ Pair wsum[ADA_THREADS / 32], csum[ROW_CLUSTER];

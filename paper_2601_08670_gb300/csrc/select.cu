@@ -55,9 +55,10 @@ __device__ __forceinline__ Cand warp_best(Cand c) {
   return c;
 }
 
+// lp, beta and r are plain pointers, as in adacad.cu: the launch before may
+// still be writing them when this one starts.
 __global__ void __cluster_dims__(SEL_CLUSTER, 1, 1) __launch_bounds__(SEL_THREADS)
-    select_dense_kernel(const float* __restrict__ lp, const float* __restrict__ beta, const float* __restrict__ r,
-                        float gamma, int N, int V, Cand* rec) {
+    select_dense_kernel(const float* lp, const float* beta, const float* r, float gamma, int N, int V, Cand* rec) {
   cg::cluster_group cluster = cg::this_cluster();
   const int b = blockIdx.y, tid = threadIdx.x, n1 = N + 1;
   __shared__ float bt[SEL_MAX_N], bias[SEL_MAX_N];
