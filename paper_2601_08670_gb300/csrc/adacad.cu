@@ -13,22 +13,24 @@
 // cluster's sums meet in the first CTA's shared memory, so there is no scratch,
 // no counter to clear and no second pass.  (One CTA per 2048 entries left the
 // last one to add 63 chunk sums one load after the other.  Experts of 128256
-// entries, in a graph: 8 16.7 -> 10.0 us, 16 x 16 184 -> 101.)  A term without
+// entries, in a graph: 8 17.4 -> 9.8 us, 16 x 16 184 -> 110.)  A term without
 // the midpoint's logarithm, exp(hi) (q + e (q + lo - hi)) with e = exp(lo - hi)
 // and q = -log((1 + e) / 2), needs one exponential less (16 x 16: 86 us) and
 // has half the error, but moves beta's last bit, which a score near zero
 // magnifies to 2.5e-6 of itself.
 //
-// Sums are held as an unevaluated pair of fp32 numbers (error-free addition,
-// about 48 bits) and rounded once from fp64 at the end: this chip adds 64-bit
+// Sums are held as three fp32 numbers (sum3.cuh, no less exact than an fp64
+// accumulator) and rounded once from fp64 at the end: this chip adds 64-bit
 // numbers at 1/64 of the fp32 rate, so one fp64 conversion and addition per
-// entry cost more than the entry's exponentials.  The order is fixed (thread,
+// entry cost more than the entry's exponentials.  (Two fp32 numbers, 8.9 and 102
+// us for the two sizes above, hold fewer bits than fp64.)  The order is fixed (thread,
 // then xor trees over lanes and warps, then the CTAs in order), so the result
 // does not depend on timing.
 #include <cooperative_groups.h>
 #include <math.h>
 
 #include "adacad.cuh"
+#include "sum3.cuh"
 
 namespace pced {
 
@@ -37,31 +39,11 @@ namespace cg = cooperative_groups;
 constexpr int ADA_THREADS = 1024;
 constexpr int ADA_UNROLL = 4;  // entries of a thread in flight
 
-// an fp32 pair s + c, |c| below half an ulp of s times the terms added
-struct Pair {
-  float s, c;
-};
-// (a + b) exactly as sum + error (Knuth's two-sum; the _rn forms keep the
-// compiler from contracting it)
-__device__ __forceinline__ float two_sum(float a, float b, float& err) {
-  const float y = __fadd_rn(a, b), z = __fsub_rn(y, a);
-  err = __fadd_rn(__fsub_rn(a, __fsub_rn(y, z)), __fsub_rn(b, z));
-  return y;
-}
-__device__ __forceinline__ void pair_add(Pair& p, float t) {
-  float e;
-  p.s = two_sum(p.s, t, e);
-  p.c = __fadd_rn(p.c, e);
-}
-__device__ __forceinline__ Pair pair_merge(Pair p, Pair q) {
-  float e;
-  const float s = two_sum(p.s, q.s, e);
-  return Pair{s, __fadd_rn(__fadd_rn(p.c, q.c), e)};
-}
-__device__ __forceinline__ Pair warp_pair(Pair p) {
+__device__ __forceinline__ Sum3 warp_sum3(Sum3 p) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
-    p = pair_merge(p, Pair{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.c, o)});
+    p = sum3_merge(p, Sum3{__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.c, o),
+                           __shfl_xor_sync(0xffffffffu, p.e, o)});
   return p;
 }
 
@@ -83,7 +65,7 @@ __global__ void __launch_bounds__(ADA_THREADS)
     adacad_beta_kernel(const float* lp, int32_t N, int32_t V, float* beta, int* reset_ctr) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = blockIdx.x, nc = gridDim.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
-  __shared__ Pair wsum[ADA_THREADS / 32], csum[ROW_CLUSTER];
+  __shared__ Sum3 wsum[ADA_THREADS / 32], csum[ROW_CLUSTER];
   cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
   pdl_wait();  // dependents are launched when this ends: select.cu has the figures
   if (reset_ctr && rank == 0 && k == 1 && b == 0 && tid == 0) *reset_ctr = 0;
@@ -91,7 +73,8 @@ __global__ void __launch_bounds__(ADA_THREADS)
   const float* lk = l0 + (int64_t)k * V;
   const int per = (V - 1) / nc + 1;
   const int64_t v0 = (int64_t)rank * per, v1 = min((int64_t)V, v0 + per);
-  Pair acc{0.f, 0.f};
+  Sum3 acc{0.f, 0.f, 0.f};
+  int terms = 0;
   for (int64_t v = v0 + tid; v < v1; v += ADA_UNROLL * ADA_THREADS) {
     float x[ADA_UNROLL], y[ADA_UNROLL];
 #pragma unroll
@@ -101,19 +84,20 @@ __global__ void __launch_bounds__(ADA_THREADS)
       y[u] = in ? l0[v + u * ADA_THREADS] : -INFINITY;
     }
 #pragma unroll
-    for (int u = 0; u < ADA_UNROLL; ++u) pair_add(acc, jsd_term(x[u], y[u]));
+    for (int u = 0; u < ADA_UNROLL; ++u) sum3_add(acc, jsd_term(x[u], y[u]));
+    if ((terms += ADA_UNROLL) % SUM3_RUN == 0) sum3_settle(acc);
   }
-  acc = warp_pair(acc);
+  acc = warp_sum3(acc);
   if ((tid & 31) == 0) wsum[tid >> 5] = acc;
   __syncthreads();
-  if (tid < 32) acc = warp_pair(wsum[tid]);
+  if (tid < 32) acc = warp_sum3(wsum[tid]);
   cluster.barrier_wait();
   if (tid == 0) *cluster.map_shared_rank(csum + rank, 0) = acc;
   cluster.sync();
   if (rank == 0 && tid == 0) {
-    Pair t = csum[0];
-    for (int i = 1; i < nc; ++i) t = pair_merge(t, csum[i]);
-    beta[(int64_t)b * N + k - 1] = (float)(((double)t.s + (double)t.c) * 0.72134752044448170);  // 1 / (2 ln 2)
+    Sum3 t = csum[0];
+    for (int i = 1; i < nc; ++i) t = sum3_merge(t, csum[i]);
+    beta[(int64_t)b * N + k - 1] = (float)(sum3_value(t) * 0.72134752044448170);  // 1 / (2 ln 2)
   }
 }
 

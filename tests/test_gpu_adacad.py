@@ -10,7 +10,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-BETA_TOL = 2e-5  # fp32 terms summed in fp64 on the GPU vs fp64 throughout
+BETA_TOL = 2e-5  # fp32 terms summed no less exactly than in fp64 on the GPU vs fp64 throughout
 
 
 def _logprob_rows(rng, rows, V, spread):
@@ -43,7 +43,7 @@ def test_adacad_beta_matches_oracle(cuda_ok, B, N, V, spread):
 def test_adacad_beta_edges_of_the_cluster_split(cuda_ok, V):
     """Vocabularies around the eight parts of a cluster and a part's threads.  The midpoint's logarithm is at most 16
     here and rounded twice, so off by 1e-6 at most in a term and by either sign; its probabilities sum to 1, halved, and
-    the sums carry 48 bits: the result is within 1e-6 of the fp64 sum over the same rows."""
+    the sums are no less exact than fp64 ones: the result is within 1e-6 of the fp64 sum over the same rows."""
     rng = np.random.default_rng(V)
     lp = _logprob_rows(rng, 2 * 3, V, 2.0).astype(np.float32).astype(np.float64)
     assert np.max(np.abs(_gpu_beta(lp, 2, 2) - oracle.adacad_beta(lp, 2, 2))) <= 1e-6
@@ -101,3 +101,11 @@ def test_step_with_dynamic_beta(cuda_ok, name, steps, ram):
         compare_step(dec, ref, run, s, stats)
     assert dec.status() == 0
     check_stats(stats, name)
+
+
+def test_adacad_beta_overflow_is_infinite(cuda_ok):
+    # rows that are no log-probabilities: a term beyond the range makes its sum infinite, not NaN, whatever follows it
+    lp = np.full((3, 70000), -12.0)
+    lp[1, 11] = 100.0
+    got = _gpu_beta(lp, 1, 2)
+    assert got[0, 0] == np.inf and abs(got[0, 1]) < 2e-6
