@@ -549,8 +549,9 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_pempty);
     const int32_t len = lens[pc.s];
+    const bool in = PCED_IN_BOUNDS(pc.s >= 0 && pc.s < S && pc.h >= 0 && pc.h < a.Hkv, a.status);
     if (pc.k0 == 0 && pc.k1 == len) {
-      if (own) {
+      if (own && in) {
         const float w = mx == -INFINITY ? 0.f : 1.f / lsum;
         float* op = a.out + ((int64_t)pc.s * a.Hq + (int64_t)pc.h * G) * D + idx0;
 #pragma unroll
@@ -565,8 +566,11 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
       *reinterpret_cast<float4*>(a.rec_o + slot * GD + idx0) = make_float4(acc[0], acc[1], acc[2], acc[3]);
       if (idx0 % D == 0) a.rec_ml[slot * G + hh] = make_float2(mx, lsum);
     }
-    if (pc.k0 == 0)  // its last key lies (p - 1 + the keys left) positions on
-      plan = make_int2(pc.s * a.Hkv + pc.h, (int)(udiv_pos(p - 1 + (len - pc.k1), per) - blockIdx.x) + 1);
+    if (pc.k0 == 0) {  // its last key lies (p - 1 + the keys left) positions on
+      const int64_t last = udiv_pos(p - 1 + (len - pc.k1), per);
+      if (in && PCED_IN_BOUNDS(last >= blockIdx.x && last < gridDim.x, a.status))
+        plan = make_int2(pc.s * a.Hkv + pc.h, (int)(last - blockIdx.x) + 1);
+    }
   }
   if (a.fused) {
     // all CTAs are one cluster: the records are there for all of them

@@ -310,7 +310,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LM_THREADS, 1)
       if (nc1) blocks(n0, half, nb1, tempty1);
       blocks(0, (nb1 & 1) ? 1 - half : half, nb0, tempty0 + 8 * b0);
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
-      if (tile < a.ntiles) fold_tile(a, tile, etid, wst, wag, wu2);  // the last pair's second half may hold no rows
+      // the last pair's second half may hold no rows
+      if (PCED_IN_BOUNDS(tile2 < ntiles, a.status) && tile < a.ntiles) fold_tile(a, tile, etid, wst, wag, wu2);
       if (!bar_sync_bounded(bar_epi, ephase, a.status)) break;
     }
   }

@@ -1,11 +1,15 @@
 """The bounds-checked build (-DPCED_BOUNDS_CHECK): every guarded global index
 (appended K/V row inside its layer region and below the capacity, partial
-record slots, residual-stream rows, LM-head record tiles, selection rows) is
-checked on the device; an index outside its buffer would set PCED_DEV_BOUNDS
-and skip the access.  On valid inputs the checked library must report no
+record slots, residual-stream rows, LM-head record tiles of both kernels,
+selection rows; of one layer's attention the segment of an output and the
+records of a cut one) is checked on the device; an index outside its buffer
+would set PCED_DEV_BOUNDS and skip the access.  On valid inputs the checked library must report no
 status bit and choose the same tokens with bit-identical hidden states as the
 release library (the checks do not touch the arithmetic).  Slab and paged
-caches, the max rule, MoE and a dynamic-beta first step are covered."""
+caches, the max rule, MoE, a dynamic-beta first step, more than 160 sequences
+(CTA pairs), one-layer attention in one and two launches and the LM head alone
+are covered; the kernels of the unfused beta and selection and of MoE / PoE hold
+no guards."""
 import json
 import os
 import subprocess
@@ -28,7 +32,7 @@ def test_checked_build_runs_clean_and_matches_release(cuda_ok):
     assert res.returncode == 0, res.stderr[-3000:]
     checked = json.loads(res.stdout.strip().splitlines()[-1])
     release = checked_run.run_cases()
-    assert len(checked) == len(release) == len(checked_run.CASES)
+    assert len(checked) == len(release) == sum(map(len, (checked_run.CASES, checked_run.ATTENTION, checked_run.LM_HEAD)))
     for c, r in zip(checked, release):
         assert c["case"] == r["case"]
         assert c["status"] == 0 and r["status"] == 0, (c, r)
