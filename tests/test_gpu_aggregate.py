@@ -50,8 +50,8 @@ def test_moe_poe_llama8(cuda_ok, rule):
     run_variant("llama8", 2, 8, aggregation=rule)
 
 
-@pytest.mark.parametrize("rule,B,N,V", [(1, 1, 1, 7), (2, 1, 5, 8191), (1, 2, 9, 1025), (2, 40, 2, 1000),
-                                        (1, 100, 4, 1023)])
+@pytest.mark.parametrize("rule,B,N,V", [(1, 1, 1, 7), (2, 1, 5, 8191), (1, 2, 9, 1025), (2, 10, 5, 1000),
+                                        (2, 40, 2, 1000), (1, 100, 4, 1023)])
 def test_moe_poe_edges_of_the_vocabulary_split(cuda_ok, rule, B, N, V):
     # vocabularies below and around a CTA's tokens, expert counts around a
     # batch of four rows, and enough (query, expert) pairs for every number

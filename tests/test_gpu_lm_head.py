@@ -64,12 +64,13 @@ def test_many_tiles_per_cta_with_two_n_chunks(cuda_ok, S):
 
 
 @pytest.mark.parametrize("S,d,V", [(96, 128, 1000), (97, 128, 1), (97, 64, 30000), (128, 192, 128), (129, 64, 129),
-                                   (160, 256, 385), (224, 64, 40000), (256, 128, 4097), (257, 64, 20001),
+                                   (160, 256, 385), (161, 128, 1128), (161, 64, 40000), (192, 320, 2049),
+                                   (193, 128, 300), (224, 64, 40000), (256, 128, 4097), (257, 64, 20001),
                                    (288, 320, 2049), (289, 128, 300), (384, 64, 9999), (385, 128, 9000),
                                    (448, 64, 700)])
 def test_pairs_of_ctas(cuda_ok, S, d, V):
-    # the row counts where a CTA pair takes over, where the columns become two
-    # chunks and where neither is double buffered; one stage per tile (d = 64)
-    # with many tiles; an odd number of 128-row tiles (the last pair's second
-    # half holds no rows)
+    # up to 160 rows one CTA takes a tile, from 161 on a pair does: around that
+    # count, where the columns become two chunks (257) and where neither is double
+    # buffered (385); one stage per tile (d = 64) with many tiles; an odd number of
+    # 128-row tiles (the last pair's second half holds no rows)
     assert run_case(S, d, V) < 1e-4
