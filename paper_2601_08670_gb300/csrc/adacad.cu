@@ -62,13 +62,12 @@ __device__ __forceinline__ float jsd_term(float a, float b) {
 // (the log-softmax pass does, in place), so its loads must not become
 // non-coherent ones, which const __restrict__ allows.
 __global__ void __launch_bounds__(ADA_THREADS)
-    adacad_beta_kernel(const float* lp, int32_t N, int32_t V, float* beta, int* reset_ctr) {
+    adacad_beta_kernel(const float* lp, int32_t N, int32_t V, float* beta) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = blockIdx.x, nc = gridDim.x, k = blockIdx.y + 1, b = blockIdx.z, tid = threadIdx.x;
   __shared__ Sum3 wsum[ADA_THREADS / 32], csum[ROW_CLUSTER];
   cluster.barrier_arrive();  // waited for before the first CTA's shared memory is written
   pdl_wait();  // dependents are launched when this ends: select.cu has the figures
-  if (reset_ctr && rank == 0 && k == 1 && b == 0 && tid == 0) *reset_ctr = 0;
   const float* l0 = lp + (int64_t)b * (N + 1) * V;
   const float* lk = l0 + (int64_t)k * V;
   const int per = (V - 1) / nc + 1;
@@ -101,11 +100,11 @@ __global__ void __launch_bounds__(ADA_THREADS)
   }
 }
 
-cudaError_t adacad_beta_launch(const float* lp, int32_t B, int32_t N, int32_t V, float* beta, int* reset_ctr, bool pdl,
+cudaError_t adacad_beta_launch(const float* lp, int32_t B, int32_t N, int32_t V, float* beta, bool pdl,
                                cudaStream_t stream) {
   const int nc = pced_host::row_cluster((int64_t)B * N);
-  return pced_host::launch_cluster(adacad_beta_kernel, dim3(nc, N, B), nc, ADA_THREADS, 0, stream, pdl, lp, N, V, beta,
-                                   reset_ctr);
+  return pced_host::launch_cluster(adacad_beta_kernel, dim3(nc, N, B), nc, ADA_THREADS, 0, stream, pdl, lp, N, V,
+                                   beta);
 }
 
 }  // namespace pced
@@ -134,7 +133,7 @@ extern "C" pced_status pced_adacad_beta(const float* logprobs, int32_t B, int32_
     return fail(PCED_ERR_WORKSPACE, "pced_adacad_beta: workspace too small or misaligned");
   if (num_sms() <= 0) return fail(PCED_ERR_NO_DEVICE, "pced_adacad_beta: no CUDA device");
   cudaStream_t s = (cudaStream_t)stream;
-  const cudaError_t e = adacad_beta_launch(logprobs, B, N, V, beta, nullptr, true, s);
+  const cudaError_t e = adacad_beta_launch(logprobs, B, N, V, beta, true, s);
   if (e != cudaSuccess) return cuda_status(e, "pced_adacad_beta launch");
   return PCED_OK;
 }

@@ -293,9 +293,9 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   if (e == cudaSuccess) e = mark();
   if (e != cudaSuccess) return cuda_status(e, "attention launch");
 
-  // dynamic contrast strength or MoE / PoE: materialise this step's
-  // log-probabilities; beta from their divergences, then either the usual
-  // fused LM head with that beta or the aggregation kernels
+  // dynamic contrast strength or MoE / PoE: materialise this step's logits
+  // (for beta their log-probabilities), beta from their divergences, then the
+  // choice from what is materialised
   const float* beta = p->beta;
   if (dyn || agg) {
     LmArgs lz = lm_args(g);
@@ -315,10 +315,9 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
       e = lm_lse_finalize_launch(W.lp, W.lm_stats, W.sel_L, S, dm.V, g.ntiles, true, !timed, s);
       if (e == cudaSuccess) e = mark();
     }
-    // the JSD kernel also re-arms the LM head's tile counter for the fused pass
     if (e == cudaSuccess && dyn) {
       ranges.next("adacad_beta");
-      e = adacad_beta_launch(W.lp, dm.B, dm.N, dm.V, p->beta_out, W.lm_tile_ctr, !timed, s);
+      e = adacad_beta_launch(W.lp, dm.B, dm.N, dm.V, p->beta_out, !timed, s);
       if (e == cudaSuccess) e = mark();
     }
     if (e != cudaSuccess) return cuda_status(e, "log-probability launches");
@@ -384,7 +383,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   la.tile_ctr = W.lm_tile_ctr;
   la.beta = beta;
   la.status = W.status;
-  la.pdl = (timed || dyn) ? 0 : LM_PDL_H;  // stage events between the launches would break the overlap
+  la.pdl = timed ? 0 : LM_PDL_H;  // stage events between the launches would break the overlap
   ranges.next("lm_head");
   e = lm_head_launch(maps, g, la, s);
   if (e == cudaSuccess) e = mark();
@@ -419,7 +418,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   sa.expert = p->expert_out;
   sa.score = p->score_out;
   sa.status = W.status;
-  sa.pdl = (timed || dyn) ? 0 : 1;
+  sa.pdl = timed ? 0 : 1;
   sa.raw_logits = p->score_mode == PCED_SCORE_LOGIT;
   ranges.next("select");
   e = select_from_records_launch(sa, s);
