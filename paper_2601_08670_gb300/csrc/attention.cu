@@ -1697,7 +1697,9 @@ static cudaError_t launch_step(const CUtensorMap& kmap, const CUtensorMap& vmap,
   cudaError_t e = set_smem_once(att_step_kernel<D, PK>, 227 * 1024, configured);
   if (e != cudaSuccess) return e;
   // every CTA waits for the others' layer results, so all must be resident at
-  // once: a cooperative launch guarantees it (or fails)
+  // once: a cooperative launch guarantees it (or fails).  Not a programmatic
+  // launch: it follows everything before it in the stream, which the LM head
+  // launched behind it relies on (LM_PDL_H)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(STEP_THREADS);

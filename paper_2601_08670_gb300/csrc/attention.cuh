@@ -96,8 +96,8 @@ cudaError_t att_layer_launch(int D, const CUtensorMap& kmap, const CUtensorMap& 
 // stores the group's sum of squares.  A piece of layer l waits for its head
 // group of x_l[s] and all group sums of x_l[s].  Everything exchanged between
 // CTAs is a tagged 64-bit word (see attention.cu).  After the last layer each
-// completing CTA writes its head group of the final hidden state; the last
-// CTA to finish advances seq_len and the epoch.
+// completing CTA writes its head group of the final hidden state.  seq_len and
+// the epoch advance near the start, by the last CTA to have read them.
 struct StepAttArgs {
   int32_t S, Hq, Hkv, G, L, n1, V, bos, max_steps;
   int64_t rows_per_layer;     // rows (of D elements) of one layer's region in the tensor maps
@@ -124,7 +124,7 @@ struct StepAttArgs {
   uint64_t* rec_o;            // [slots][G*D] tagged partial outputs
   uint64_t* rec_ml;           // [slots][G][2] tagged (max, sum)
   int32_t* epoch;             // [1] launches completed (tags name the launch)
-  int32_t* done_cnt;          // [1] CTAs finished (zero between launches)
+  int32_t* done_cnt;          // [1] CTAs that have read the lengths and the epoch (zero between launches)
   __nv_bfloat16* hidden;      // [S][d] final hidden state
   __nv_bfloat16* hidden_copy; // optional copy of `hidden`
   unsigned long long wait_ns; // limit of the kernel's waits on other warps and CTAs (PCED_DEV_TIMEOUT after it)

@@ -120,8 +120,8 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // of these instructions live in uniform registers, and in code that a single
 // lane runs alone each one is moved there again for every instruction (an MMA
 // cost 93-170 clocks of issue, with this form 37, against the 64 that M = 128,
-// N = 128 takes to execute; the LM head at 33 hidden rows went from 170 to 162
-// us a call, at 272 rows on CTA pairs from 355 to 272).
+// N = 128 takes to execute; when it was introduced the LM head at 33 hidden rows
+// went from 170 to 162 us a call, at 272 rows on CTA pairs from 355 to 272).
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t on;
   asm volatile(
@@ -472,10 +472,6 @@ pced_status make_tmap_2d(CUtensorMap* map, const void* base, uint64_t rows, uint
                          uint32_t box_cols, bool l2_promote_256);
 pced_status make_tmap_kv(CUtensorMap* map, const void* base, uint64_t rows, uint32_t D, uint32_t box_rows);
 
-// Launch a kernel, with pdl as a programmatic dependent of the stream's previous
-// kernel.  Every kernel launched so calls pdl_wait() in all of its threads
-// before it touches memory that an earlier launch may write or still read, so
-// only its launch, and what it does before the wait, overlap that kernel.
 // CTAs per (query, expert) of the kernels that read an expert's and the
 // amateur's row of the vocabulary: a cluster of up to ROW_CLUSTER, fewer from
 // two CTAs per SM on, where a longer part of the row per CTA pays for its
@@ -484,6 +480,16 @@ pced_status make_tmap_kv(CUtensorMap* map, const void* base, uint64_t rows, uint
 // 41 with two).
 int row_cluster(int64_t rows);
 
+// Launch a kernel, with pdl as a programmatic dependent of the stream's previous
+// kernel: only its launch, and what it does before pdl_wait(), overlap that
+// kernel.  The kernels launched so call pdl_wait() in all of their threads
+// before they touch memory that an earlier launch may write or still read, and
+// read it with plain loads (not non-coherent ones).  The two LM heads alone
+// differ: their TMA warp waits (LM_PDL_ALL: before its first copy; LM_PDL_H:
+// before its first copy of H), and the other warps are behind it, since all that
+// they write follows from its copies.  What they touch before that wait, beta,
+// W and the tile counter, must not be written by the launch before: see
+// LM_PDL_H in lm_head.cuh.
 template <typename... P>
 cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int cluster, unsigned threads, size_t smem,
                            cudaStream_t stream, bool pdl, P... args) {

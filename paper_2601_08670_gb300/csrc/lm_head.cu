@@ -388,10 +388,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
-  // the log-softmax or aggregation kernels come at the end: beside this one
-  // their CTAs only wait (S = 272 252 -> 247 us a call, S = 33, d = 1024, V = 50000
-  // 29.1 -> 27.4); the selection's cluster, which starts later, comes early
-  // (the 9-row step 538 us, 543 with a late one)
+  // the log-softmax or aggregation kernels come at the end (at the start, a call
+  // in a graph takes 250 us instead of 245 at S = 272, 24.4 instead of 23.0 at S =
+  // 33, d = 1024, V = 50000); the selection's cluster, which starts later, comes
+  // early (the 9-row step 538 us, 543 with a late one)
   if (a.mode == 0) pdl_launch_dependents();
   if (warp == 1) {
     tc_fence_after();
@@ -453,11 +453,13 @@ __global__ void __launch_bounds__(LSE_THREADS) lm_lse_kernel(const float2* rec_s
 }
 
 // CTA (chunk, row s), all rows of the last chunk first (the tiles written last
-// are still in L2: 258 us instead of 276 for the whole call at S = 272, V =
-// 128256): chunk of logits -> log-probabilities in place.  FUSED: every CTA of
-// row s also forms lse[s], one launch less (1.5 us at S = 9); otherwise
-// lm_lse_kernel has written it, so that a CTA's time is that of its loads and
-// stores alone (258 us instead of 266 at S = 272, equal at S = 65).
+// are still in L2: the whole call, in a graph, 245 us instead of 261 at S = 272, V
+// = 128256): chunk of logits -> log-probabilities in place.  FUSED: every CTA of
+// row s also forms lse[s], one launch less (6.8 us instead of 7.2 at S = 3, d =
+// 512, V = 8192, 23.0 instead of 23.7 at S = 33, d = 1024, V = 50000; not at S = 9,
+// V = 128256: 162.9, 161.6); otherwise lm_lse_kernel has written it, so that a
+// CTA's time is that of its loads and stores alone (245 us instead of 256 at S =
+// 272, 185.6 instead of 190.4 at S = 128, 168.1 instead of 170.0 at S = 65).
 template <bool FUSED, int CHUNK>
 __global__ void __launch_bounds__(LSE_THREADS) lm_lse_finalize_kernel(float* logits, const float2* rec_stats, float* lse,
                                                                       int32_t S, int32_t V, int32_t nrec) {

@@ -16,8 +16,14 @@ constexpr int LM_TRING = 32;     // claimed-tile ring between the TMA and the ot
 constexpr int LM_A_BYTES = LM_TILE_V * LM_TILE_K * 2;  // 16 KB
 constexpr size_t LM_SMEM_BUDGET = 227 * 1024;
 // From this many hidden rows on a tile is taken by a pair of CTAs
-// (lm_head_pair.cu), below by one (lm_head.cu): equal at 128 rows, 207 against
-// 205 us at 160, 219 against 216 us at 192 (d = 4096, V = 128256).
+// (lm_head_pair.cu), below by one (lm_head.cu), which TMEM allows up to 256 rows.
+// One CTA / pairs, us a call in a graph: d = 4096, V = 128256 185 / 185 at 128
+// rows, 198 / 194 at 160, 209 / 203 at 192, 248 / 232 at 256; d = 4096, V = 8000
+// 27.4 / 27.1, 28.5 / 29.4, 35.1 / 34.5 at 160, 192, 256; d = 1792, V = 30000 36.2 /
+// 37.0 and 42.2 / 42.0 at 192 and 256.  The line is drawn for such rows; with
+// shorter ones one CTA stays ahead up to 256 rows, which the rule leaves: d =
+// 1024, V = 50000 40.8 / 44.4 and 50.1 / 52.2 at 192 and 256, d = 512, V = 8192 14.8 /
+// 16.8 and 17.4 / 19.1, d = 64 at most 14 % more.
 constexpr int LM_PAIR_MIN_S = 161;
 
 struct LmGeom {
@@ -29,7 +35,12 @@ struct LmGeom {
 // returns false when the shape is unsupported
 bool lm_geometry(int32_t S, int32_t d, int32_t V, LmGeom* g);
 
-constexpr int LM_PDL_H = 1;    // of the kernel that writes H: the weights are read before it ends
+// Of the kernel that writes H: the weights are read, tiles claimed and beta's
+// coefficients formed before it ends.  That kernel must write none of these, and
+// must itself be launched in full stream order (att_step_launch is), so that
+// the selection before it has reset the tile counter and any upload of beta has
+// landed.
+constexpr int LM_PDL_H = 1;
 constexpr int LM_PDL_ALL = 2;  // of any kernel: nothing is read before it ends
 
 struct LmArgs {

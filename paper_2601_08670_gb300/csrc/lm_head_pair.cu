@@ -16,17 +16,17 @@
 // second one first, so the next tile's MMAs wait for n1 columns of it only.
 //
 // W comes from HBM, H from L2, so they have rings of their own: five stages of
-// H, and W in the rest of shared memory (one ring of both, with three stages:
-// 268 against 264 us a call at S = 272; two stages of H: 312, four: 273 against
-// 265 with five).  An epilogue warp gives its columns back as soon as they
-// are in its registers (265 -> 257 us).
+// H, and W in the rest of shared memory (S = 272, a call in a graph: two stages
+// of H 285 us, three 256, four 248, five 245, six 246; one ring of both with three
+// stages was 4 us slower than two rings).  An epilogue warp gives its columns back
+// as soon as they are in its registers (8 us less).
 //
-// Measured (pced_lm_head_logprobs, d = 4096, V = 128256; one CTA per tile ->
-// pairs): S = 272 370 -> 257 us, S = 384 509 -> 345, S = 512 583 -> 462; in a
-// decode step of 272 sequences 358 -> 207 us.  About half of that came from
-// issuing MMAs and copies in warp-uniform code (elect_one in common.cuh), which
-// lm_head.cu has too: with it one CTA per tile is as fast up to 128 rows (192
-// us), 207 against 205 us at 160 and 254 against 239 at 256.
+// Measured (pced_lm_head_logprobs, d = 4096, V = 128256, in a graph; one CTA per
+// tile -> pairs): S = 272 369 -> 245 us, S = 384 508 -> 344, S = 512 581 -> 456; a
+// call among others, on new inputs, at S = 272 372 -> 263; the launch in a decode
+// step of 272 sequences 358 -> 207.  About half of that came from issuing MMAs
+// and copies in warp-uniform code (elect_one in common.cuh), which lm_head.cu
+// has too; LM_PAIR_MIN_S in lm_head.cuh has both kernels where one CTA can do.
 //
 // Roles per CTA as in lm_head.cu.  CTA 0 of the pair claims tiles (both CTAs get
 // them through a ring in shared memory), waits for the operands of both (its

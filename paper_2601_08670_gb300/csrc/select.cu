@@ -15,10 +15,11 @@
 // CTAs share a chunk (their bests meet in the first one's shared memory, so
 // the workspace still holds one record per SEL_CHUNK tokens), and the second
 // kernel's launch is set up beside the first (programmatic launch).  Neither
-// this kernel nor adacad.cu's triggers its dependents early: CTAs that only
-// wait would hold the slots of its own later ones (beta, select and relevance
-// in a graph, us: 33 rows of V = 128256 34.4 -> 25.1, 9 rows 16.3 -> 15.7,
-// 4 x 9 rows of V = 50000 18.8 -> 16.3).
+// this kernel nor adacad.cu's triggers its dependents early; with a trigger at
+// their start beta, select and relevance in a graph took longer, us: 33 rows of
+// V = 128256 34.4 against 25.1, 9 rows 16.3 against 15.7, 4 x 9 rows of V = 50000
+// 18.8 against 16.3 (the dependents start once every CTA is running and then
+// share the SMs with them; what of that costs the time was not taken apart).
 #include <cooperative_groups.h>
 #include <math.h>
 

@@ -24,7 +24,7 @@ namespace pced {
 struct StepLayout {
   int* status;
   int32_t* done_counter;  // selection kernel: queries finished this step
-  int32_t* att_done;      // attention: CTAs finished
+  int32_t* att_done;      // attention: CTAs that have read the lengths
   int32_t* att_epoch;     // attention: launches completed
   int32_t* lm_tile_ctr;   // LM head: vocabulary tiles claimed (reset by the selection)
   float* sel_L;           // log-sum-exps of the rows (dynamic beta, MoE / PoE)
@@ -311,6 +311,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
     // read the raw logits and form the rows' log-sum-exps themselves); beta
     // needs the normalised rows
     if (e == cudaSuccess && dyn) {
+      // (one launch at any number of rows, as the launch list says)
       ranges.next("lse_finalize");
       e = lm_lse_finalize_launch(W.lp, W.lm_stats, W.sel_L, S, dm.V, g.ntiles, true, !timed, s);
       if (e == cudaSuccess) e = mark();
