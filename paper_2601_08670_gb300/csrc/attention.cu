@@ -811,14 +811,16 @@ __device__ __forceinline__ void cursor_next(TileCursor<PAGED>& c, const StepAttA
 }
 
 // The producer: K/V tiles of every layer in consumption order into the
-// NST-stage ring; the L2 prefetch cursor runs pf_tiles ahead so HBM keeps
-// streaming while the ring is full, ATT_PF_FIRST more at first, while the
-// consumers wait for the launch's first queries.  The ring is filled before
-// the first prefetch: with the prefetches first, the first tile was asked for
-// 8 us after the start of a 32-layer launch instead of 4 (attention of four
-// layers of 9 x 2080 rows 69 -> 67 us, 28 layers of 17 x 4128 rows, 4 kv-heads, 598
-// -> 593).  One thread.
-constexpr int ATT_PF_FIRST = 4;
+// NST-stage ring; the L2 prefetch cursor runs pf_tiles ahead of the ring so HBM
+// keeps streaming while it is full.  The ring is filled before the first
+// prefetch: with the prefetches first, the first tile was asked for 8 us after
+// the start of a 32-layer launch instead of 4.  The loop after that does the same
+// for every tile, one load and one prefetch: the thread's time per tile is close
+// to a tile's share of the bandwidth, the more so with paged caches, whose
+// cursors look up blocks.  (32 layers of 9 x 2080 rows, attention of a step, six
+// tiles ahead: 256-row blocks 403 us, 440 with the ring's start and a counted
+// number of prefetches in the one loop, 407 with the prefetches first; 64-row
+// blocks 430, 469, 432; slabs 381, 381, 383.)  One thread.
 template <int D, bool PAGED>
 __device__ __forceinline__ void produce_tiles(const CUtensorMap* kmap, const CUtensorMap* vmap, const StepAttArgs& a,
                                               const int64_t* pre, const int32_t* lens, const GroupPlan& gp,
@@ -826,16 +828,11 @@ __device__ __forceinline__ void produce_tiles(const CUtensorMap* kmap, const CUt
                                               uint32_t bar_full, uint32_t bar_empty) {
   using C = AttCfg<D>;
   const uint64_t pol = policy_evict_first();
-  TileCursor<PAGED> ld, pf;
+  TileCursor<PAGED> ld;
   cursor_begin(ld, a, pre, lens, gp, D, ptab, ptab_n);
   uint32_t it = 0, st = 0, ph = 0;
-  int ahead = 0;  // tiles prefetched past the loaded ones
   bool ok = true;
-  while (ld.ok) {
-    if (!mbar_wait(bar_empty + 8 * st, ph ^ 1u, a.status, a.wait_ns)) {
-      ok = false;
-      break;
-    }
+  auto load = [&]() {
     const uint32_t fb = bar_full + 8 * st;
     const uint32_t sk = base + st * C::STAGE_BYTES, sv = sk + C::TILE_BYTES;
     mbar_arrive_expect_tx(fb, C::STAGE_BYTES);
@@ -848,21 +845,27 @@ __device__ __forceinline__ void produce_tiles(const CUtensorMap* kmap, const CUt
       ph ^= 1u;
     }
     cursor_next(ld, a, pre, lens, gp, D, ptab, ptab_n);
-    --ahead;
-    // the ring is filled first; then the prefetch runs ahead of it
-    if (it < NST) continue;
-    if (it == NST) {
-      pf = ld;
-      ahead = 0;
+  };
+#pragma unroll 1
+  while (ld.ok && it < NST) load();
+  TileCursor<PAGED> pf = ld;
+  pf.ok = ld.ok && a.pf_tiles > 0;
+  auto prefetch = [&]() {
+    if (!pf.bad) {
+      tma_prefetch_l2_3d(kmap, 0, pf.tile_row(), 0);
+      tma_prefetch_l2_3d(vmap, 0, pf.tile_row(), 0);
     }
-    const int want = a.pf_tiles + (it == NST && a.pf_tiles > 0 ? ATT_PF_FIRST : 0);
-    for (; ahead < want && pf.ok; ++ahead) {
-      if (!pf.bad) {
-        tma_prefetch_l2_3d(kmap, 0, pf.tile_row(), 0);
-        tma_prefetch_l2_3d(vmap, 0, pf.tile_row(), 0);
-      }
-      cursor_next(pf, a, pre, lens, gp, D, ptab, ptab_n);
+    cursor_next(pf, a, pre, lens, gp, D, ptab, ptab_n);
+  };
+#pragma unroll 1
+  for (int i = 0; i < a.pf_tiles && pf.ok; ++i) prefetch();
+  while (ld.ok) {
+    if (!mbar_wait(bar_empty + 8 * st, ph ^ 1u, a.status, a.wait_ns)) {
+      ok = false;
+      break;
     }
+    load();
+    if (pf.ok) prefetch();
   }
   if (!ok) {
     for (uint32_t j = (it >= NST ? it - NST : 0); j < it; ++j)
@@ -1619,7 +1622,11 @@ static int env_int(const char* name, int dflt, int lo, int hi) {
   return v < lo ? lo : (v > hi ? hi : v);
 }
 int att_step_seg_cost(int D) { return env_int("PCED_ATT_SEGCOST", 512, 0, 1 << 20); }
-int att_step_pf_tiles() { return env_int("PCED_ATT_PF", 6, 0, 64); }
+// Six tiles ahead of the ring with slab caches (a 32-layer step of 9 sequences 531
+// us, 534 with four; more thrash the L2), three with paged ones, whose blocks lie
+// scattered: against six, 272 sequences of 64-row blocks 1131 and 1163 us (six
+// layers), 33 ragged sequences 1 % less, 9 sequences within 1 % either way.
+int att_step_pf_tiles(bool paged) { return env_int("PCED_ATT_PF", paged ? 3 : 6, 0, 64); }
 // Two groups, the second of which streams while the first one's layer dependency
 // resolves (eight layers of 9 sequences of 2080 rows: 120 us against 137 with
 // one).  Two also where segments are many more than CTAs, so that few are split

@@ -135,7 +135,7 @@ int64_t att_step_slots(int32_t S, int32_t Hkv);
 // tuning of the partition and the prefetch distance (PCED_ATT_SEGCOST /
 // PCED_ATT_PF in the environment override the defaults)
 int att_step_seg_cost(int D);
-int att_step_pf_tiles();
+int att_step_pf_tiles(bool paged);
 int att_step_groups();
 int att_step_seg_lead(int seg_cost);
 cudaError_t att_step_launch(int D, const CUtensorMap& kmap, const CUtensorMap& vmap, const StepAttArgs& a, int ctas,

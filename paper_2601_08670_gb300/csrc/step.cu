@@ -251,7 +251,7 @@ extern "C" pced_status pced_step(const pced_step_args* p, void* stream) {
   at.scale_log2 = p->attn_scale * 1.4426950408889634f;
   at.rms_eps = p->rms_eps;
   at.seg_cost = att_step_seg_cost(dm.D);
-  at.pf_tiles = att_step_pf_tiles();
+  at.pf_tiles = att_step_pf_tiles(paged);
   at.groups = att_step_groups();
   at.seg_lead = att_step_seg_lead(at.seg_cost);
   if (paged) {
