@@ -24,7 +24,7 @@
 // Measured (pced_lm_head_logprobs, d = 4096, V = 128256, in a graph; one CTA per
 // tile -> pairs): S = 272 369 -> 245 us, S = 384 508 -> 344, S = 512 581 -> 456; a
 // call among others, on new inputs, at S = 272 372 -> 263; the launch in a decode
-// step of 272 sequences 358 -> 207-221 (the clock that the box's power leaves).  About half of that came from issuing MMAs
+// step of 272 sequences 358 -> 207-221 (by the clock that the power limit leaves).  About half of that came from issuing MMAs
 // and copies in warp-uniform code (elect_one in common.cuh), which lm_head.cu
 // has too; LM_PAIR_MIN_S in lm_head.cuh has both kernels where one CTA can do.
 //
